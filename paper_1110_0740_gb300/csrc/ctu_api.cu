@@ -389,6 +389,13 @@ static StepArgs make_args(const ctu_ctx *ctx, const double *Uin, double *Uout, i
     a.igm = tm ? 0.0 : 1.0 / (ctx->cfg.gamma - 1.0);
     a.gamf = (float)a.gam;
     a.gm1f = tm ? 0.0f : (float)(ctx->cfg.gamma - 1.0);
+    if (ctx->cfg.physics == CTU_SRMHD && !tm) {
+        const double ig = ctx->cfg.gamma / (ctx->cfg.gamma - 1.0), g1 = (ctx->cfg.gamma - 1.0) / ctx->cfg.gamma;
+        a.sr_g1h = (float)g1;
+        a.sr_g1l = (float)(g1 - (double)a.sr_g1h);
+        a.sr_igh = (float)ig;
+        a.sr_igl = (float)(ig - (double)a.sr_igh);
+    }
     a.glm_alpha = ctx->cfg.glm_alpha;
     a.upwind = ctx->cfg.trace_mode;
     a.limiter = ctx->cfg.recon;

@@ -32,6 +32,7 @@
 #include "df.cuh"
 #include "mhd_device.cuh"
 #include "srmhd_device.cuh"
+#include "sr_df.cuh"
 
 namespace ctu {
 
@@ -69,6 +70,9 @@ struct StepArgs {
     double gam;
     double igm;            // 1/(Gamma-1)
     float gamf, gm1f;      // Gamma, Gamma-1 in float
+    // relativistic ideal gas: (Gamma-1)/Gamma and its inverse as double-float
+    // pairs (0 with the Taub-Mathews equation of state)
+    float sr_g1h, sr_g1l, sr_igh, sr_igl;
     double glm_alpha;
     int upwind;            // tracing mode (CTU_TRACE_*); 2 and 3 only in the reference-state kernels
     int limiter;           // linear reconstruction's slope (CTU_LINEAR_*), RECON_LIN kernels
@@ -399,11 +403,37 @@ __device__ __forceinline__ unsigned int prim_any(const double (&U)[NV], const St
         return ok ? 0u : state_flags(Vd[0], Vd[4]);
     }
     if (PHYS == PH_MHD) return prim_of<R>(U, a, V);
-    double Vd[NV];
-    const unsigned int st = sr_prim<R>(U, a.gam, Vd);
+    if constexpr (PHYS == PH_SR && sizeof(R) == 4) {
+        SrState u;
+        u.D = sr_split(U[0]);
+        u.tau = d_add(sr_split(U[4]), u.D);
 #pragma unroll
-    for (int q = 0; q < NV; ++q) V[q] = (R)Vd[q];
-    return st;
+        for (int k = 0; k < 3; ++k) {
+            u.m[k] = sr_split(U[1 + k]);
+            u.b[k] = sr_split(U[5 + k]);
+        }
+        float v[5];
+        if (a.sr_g1h > 0.0f && sr_recover(u, 0.0f, df{a.sr_g1h, a.sr_g1l}, v)) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q) V[q] = v[q];
+#pragma unroll
+            for (int q = 5; q < NV; ++q) V[q] = d2f_int(U[q]);
+            return 0u;
+        }
+        SrCons c;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) c.U[q] = U[q];
+        const SrOut o = sr_prim_slow(c, a.gam, 0.0);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) V[q] = o.V[q];
+        return o.st;
+    } else {
+        double Vd[NV];
+        const unsigned int st = sr_prim<R>(U, a.gam, Vd);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) V[q] = (R)Vd[q];
+        return st;
+    }
 }
 
 // CFL speed of one cell: max_d (largest |signal speed| along d) / dx_d.
@@ -509,24 +539,36 @@ __device__ __forceinline__ unsigned int interface_state(const R (&W)[NV], const 
     }
 }
 
+// Sweeps whose recoveries run in double-float (sr_df.cuh).  The others keep the
+// float64 iteration inline: their float32 fluxes are compiled around it, and
+// another shape of that code moves the fused multiply-adds the compiler picks
+// in them, hence the last bit of every flux.
+__host__ __device__ constexpr bool sr_df_sweep(int D) { return D == 0; }
+
 // SRMHD interface state at n+1/2: U(V*) + T formed in float64, recovered by
 // the float64 Newton iteration (Eq. transv).
-template <class R>
+template <class R, int D>
 __device__ __forceinline__ unsigned int sr_interface(const R (&W)[NV], const R (&T)[NV], const StepArgs &a,
                                                      R (&out)[NV])
 {
-    double U[NV], V[NV];
-    sr_cons<double, R>(W, a.gam, U);
-    // Newton starts from the W of the predicted state V* (the transverse
-    // correction T is an O(dt) change)
-    const double v2 = (double)W[1] * W[1] + (double)W[2] * W[2] + (double)W[3] * W[3];
-    const double W0 = sr_w<double>((double)W[0], (double)W[4], a.gam) * rcp64(1.0 - v2);
+    if constexpr (sizeof(R) == 4 && sr_df_sweep(D)) {
+        SrFace f;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) U[q] += (double)T[q];
-    const unsigned int st = sr_prim<R>(U, a.gam, V, W0);
+        for (int q = 0; q < NV; ++q) {
+            f.V[q] = W[q];
+            f.T[q] = T[q];
+        }
+        const SrOut o = sr_interface_call(f, df{a.sr_g1h, a.sr_g1l}, df{a.sr_igh, a.sr_igl}, a.gam);
 #pragma unroll
-    for (int q = 0; q < NV; ++q) out[q] = (R)V[q];
-    return st;
+        for (int q = 0; q < NV; ++q) out[q] = o.V[q];
+        return o.st;
+    } else {
+        double V[NV];
+        const unsigned int st = sr_interface64<R>(W, T, a.gam, V);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) out[q] = (R)V[q];
+        return st;
+    }
 }
 
 // Trace one cell along D: stencil (local order) -> interface states (global).
@@ -564,11 +606,16 @@ __device__ __forceinline__ unsigned int trace_cell_t(const StepArgs &a, const De
         char_predict<R, PPM>(vs, pgam<R>(a), ch, dtdx, a.upwind, lim,
                              PPM == RECON_WENO3 ? R(P.dx[D] * P.dx[D]) : R(0), pl, ml);
     } else {
-        double U0[NV];
         const long long gi = P.base + (c - P.soff);
+        if constexpr (sizeof(R) == 4 && sr_df_sweep(D)) {
+            f |= sr_mh_predict_f(vs[1], vs[2], vs[3], a.U + gi, a.ustride, [](int q) { return gperm<D>(q); },
+                                 pgam<R>(a), ch, dtdx, a.gam, df{a.sr_g1h, a.sr_g1l}, df{a.sr_igh, a.sr_igl}, pl, ml);
+        } else {
+            double U0[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) U0[q] = a.U[gperm<D>(q) * a.ustride + gi];
-        f |= sr_mh_predict<R>(vs[1], vs[2], vs[3], U0, pgam<R>(a), ch, dtdx, a.gam, pl, ml);
+            for (int q = 0; q < NV; ++q) U0[q] = a.U[gperm<D>(q) * a.ustride + gi];
+            f |= sr_mh_predict<R>(vs[1], vs[2], vs[3], U0, pgam<R>(a), ch, dtdx, a.gam, pl, ml);
+        }
     }
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -579,8 +626,8 @@ __device__ __forceinline__ unsigned int trace_cell_t(const StepArgs &a, const De
         f |= interface_state<R, IFACE64>(pg, Tc, a, Vp);
         f |= interface_state<R, IFACE64>(mg, Tc, a, Vm);
     } else {
-        f |= sr_interface<R>(pg, Tc, a, Vp);
-        f |= sr_interface<R>(mg, Tc, a, Vm);
+        f |= sr_interface<R, D>(pg, Tc, a, Vp);
+        f |= sr_interface<R, D>(mg, Tc, a, Vm);
     }
     return f;
 }

@@ -1,0 +1,469 @@
+// sr_df.cuh -- the relativistic primitive recovery of the mixed path in
+// double-float arithmetic, with a certificate that the float32 result is the
+// one the float64 iteration (sr_prim_mixed) rounds to.
+//
+// Why: the recovery needs float64 (W cancels against rho gamma and B^2 in the
+// energy equation), and GB300 issues 2 float64 operations per SM and cycle
+// against 128 of float32, so eleven float64 recoveries per cell and step held
+// the whole path at the FP64 pipe (85% busy, the FMA pipe below 3%).  A
+// double-float operation is 6 to 20 float32 ones: about a fifth of a float64
+// operation's share of its pipe.  Measured at 256^3 (beam, mixed): k_prim
+// 7.15 -> 1.30 ms, the x sweep 56.1 -> 15.4 ms.  Only the five float32 values rho, v, p leave
+// a recovery, so double-float (~2^-46) decides their rounding for all but
+// the few lanes whose value lies within the arithmetic's error of a rounding
+// boundary.  Those lanes, and every state that is not plainly physical, take
+// the float64 iteration instead (the callers' noinline slow paths), so that
+// every result is the float64 iteration's, bit for bit.
+//
+// The iterates follow sr_prim_mixed's: the same float32 Newton steps from the
+// same guess, then its float64 steps in double-float, with the first-order
+// carry of v^2 and p to the last W.  v^2 and its derivative are written
+// without the quotient N / D: with t = S/W,
+//   v^2 = (m^2 + t^2 (2W + B^2)) / (W + B^2)^2,
+//   dv^2/dW = -2 (v^2 + t^2/W) / (W + B^2).
+//
+// Error of the operations, in units of 2^-48 relative (u^2, u = 2^-24; Joldes,
+// Muller & Popescu, "Tight and rigorous error bounds for basic building
+// blocks of double-word arithmetic", ACM TOMS 2017): sum 3, product 5 to 7,
+// reciprocal and reciprocal square root about 4.  All are explicitly rounded:
+// a multiplication fused into a following addition would break the
+// error-free transformations.
+#pragma once
+
+#include "srmhd_device.cuh"
+
+namespace ctu {
+
+__device__ __forceinline__ df d_two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b);
+    const float bb = __fadd_rn(s, -a);
+    return df{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+__device__ __forceinline__ df d_norm(float a, float b)  // |a| >= |b|
+{
+    const float s = __fadd_rn(a, b);
+    return df{s, __fadd_rn(b, -__fadd_rn(s, -a))};
+}
+__device__ __forceinline__ df d_two_prod(float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    return df{p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ df d_neg(df x) { return df{-x.hi, -x.lo}; }
+__device__ __forceinline__ df d_half(df x) { return df{__fmul_rn(0.5f, x.hi), __fmul_rn(0.5f, x.lo)}; }
+__device__ __forceinline__ df d_add(df x, df y)  // either signs
+{
+    df s = d_two_sum(x.hi, y.hi);
+    const df t = d_two_sum(x.lo, y.lo);
+    s = d_norm(s.hi, __fadd_rn(s.lo, t.hi));
+    return d_norm(s.hi, __fadd_rn(s.lo, t.lo));
+}
+__device__ __forceinline__ df d_addp(df x, df y)  // operands of one sign
+{
+    const df s = d_two_sum(x.hi, y.hi);
+    return d_norm(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
+}
+__device__ __forceinline__ df d_addf(df x, float y)
+{
+    const df s = d_two_sum(x.hi, y);
+    return d_norm(s.hi, __fadd_rn(s.lo, x.lo));
+}
+__device__ __forceinline__ df d_mul(df x, df y)
+{
+    const df p = d_two_prod(x.hi, y.hi);
+    return d_norm(p.hi, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p.lo)));
+}
+__device__ __forceinline__ df d_mulf(df x, float y)
+{
+    const df p = d_two_prod(x.hi, y);
+    return d_norm(p.hi, __fmaf_rn(x.lo, y, p.lo));
+}
+__device__ __forceinline__ df d_sqr(df x)
+{
+    const df p = d_two_prod(x.hi, x.hi);
+    return d_norm(p.hi, __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, p.lo));
+}
+// 1/y: a float32 seed r and its residual e = 1 - y r to second order.
+__device__ __forceinline__ df d_rcp(df y)
+{
+    const float r = __fdividef(1.0f, y.hi);
+    const float e = __fmaf_rn(-y.lo, r, __fmaf_rn(-y.hi, r, 1.0f));
+    return d_norm(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+// 1/sqrt(x): a float32 seed y and its residual e = 1 - x y^2 to second order.
+__device__ __forceinline__ df d_rsqrt(df x)
+{
+    const float y = rsqrtf(x.hi);
+    const df t = d_mul(x, d_two_prod(y, y));
+    const float e = __fadd_rn(__fadd_rn(1.0f, -t.hi), -t.lo);
+    return d_norm(y, __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f))));
+}
+
+// Whether every value within d of x rounds to x.hi (false for a nan).
+__device__ __forceinline__ bool d_certain(df x, float d)
+{
+    return __fadd_rn(x.hi, __fadd_rn(x.lo, d)) == x.hi && __fadd_rn(x.hi, __fadd_rn(x.lo, -d)) == x.hi;
+}
+
+// float64 -> float32, round to nearest even, by integer operations (values
+// below the normal float range become signed zeros, as under -ftz).
+__device__ __forceinline__ float d2f_int(double x)
+{
+    const int hw = __double2hiint(x);
+    const unsigned lw = (unsigned)__double2loint(x);
+    const int e = (hw >> 20) & 0x7FF;
+    const unsigned sign = (unsigned)hw & 0x80000000u;
+    if (e < 1023 - 126) return __uint_as_float(sign);
+    if (e > 1023 + 127) {
+        const bool nan = e == 0x7FF && ((((unsigned)hw & 0xFFFFFu) | lw) != 0u);
+        return __uint_as_float(sign | 0x7F800000u | (nan ? 0x400000u : 0u));
+    }
+    unsigned m = ((unsigned)(e - 1023 + 127) << 23) | (((unsigned)hw & 0xFFFFFu) << 3) | (lw >> 29);
+    const unsigned rem = lw & 0x1FFFFFFFu;
+    m += (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
+    return __uint_as_float(sign | m);
+}
+
+// A conserved state for the recovery: D, tau = E + D, m, B.
+struct SrState {
+    df D, tau, m[3], b[3];
+};
+
+// 1 - v^2 of a float32 state, formed from the largest component as
+// (1 - |v|)(1 + |v|) less the other squares, so that a fast flow along an axis
+// loses nothing in it; and W = w gamma^2 (ideal gas; ig1: Gamma / (Gamma - 1)).
+__device__ __forceinline__ void sr_w_of(const float (&V)[9], df ig1, df &ev, df &W)
+{
+    const float ax = fabsf(V[1]), ay = fabsf(V[2]), az = fabsf(V[3]);
+    const float big = fmaxf(ax, fmaxf(ay, az));
+    const float s1 = ax == big ? ay : ax, s2 = ax == big ? az : (ay == big ? az : ay);
+    ev = d_add(d_mul(d_two_sum(1.0f, -big), d_two_sum(1.0f, big)),
+               d_neg(d_addp(d_two_prod(s1, s1), d_two_prod(s2, s2))));
+    W = d_mul(d_addf(d_mulf(ig1, V[4]), V[0]), d_rcp(ev));
+}
+
+// U(V) + T of a float32 state for sr_recover; W0: its w gamma^2.
+__device__ __forceinline__ void sr_state_of(const float (&V)[9], const float (&T)[9], df ig1, SrState &u, float &W0)
+{
+    df ev, W;
+    sr_w_of(V, ig1, ev, W);
+    W0 = W.hi;
+    const df B2 = d_addp(d_addp(d_two_prod(V[5], V[5]), d_two_prod(V[6], V[6])), d_two_prod(V[7], V[7]));
+    const df vB = d_add(d_add(d_two_prod(V[1], V[5]), d_two_prod(V[2], V[6])), d_two_prod(V[3], V[7]));
+    const df Wb = d_addp(W, B2);
+    u.D = d_addf(d_mulf(d_rsqrt(ev), V[0]), T[0]);
+    // W - p + (B^2 (1 + v^2) - (v.B)^2) / 2, with 1 + v^2 = 2 - (1 - v^2)
+    const df q = d_add(d_mul(B2, d_addf(d_neg(ev), 2.0f)), d_neg(d_sqr(vB)));
+    u.tau = d_add(d_add(d_addf(W, -V[4]), d_half(q)), d_two_sum(T[4], T[0]));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        u.m[k] = d_addf(d_add(d_mulf(Wb, V[1 + k]), d_neg(d_mulf(vB, V[5 + k]))), T[1 + k]);
+        u.b[k] = d_two_sum(V[5 + k], T[5 + k]);
+    }
+}
+
+// Error bounds of sr_recover, in units of 2^-48: K times the sums of the
+// magnitudes that enter 1 - v^2, the energy equation and the velocities.
+// With all three K = 1 no value out of 2e7 beam, ambient, magnetised and
+// random states rounded differently from the float64 iteration's (with 0.3,
+// 2e-5 of them did); K = 3 leaves 0.4% of the beam's and 0.1% of the
+// ambient's states to the float64 path.
+constexpr float SR_MARGIN = 1.0f / 281474976710656.0f;  // 2^-48
+#ifndef SR_K
+#define SR_K 3.0f
+#endif
+constexpr float SR_K_EV = SR_K, SR_K_F = SR_K, SR_K_V = SR_K;
+
+// W from the energy equation in float32, as sr_prim64's bracketed iteration:
+// an upper bound by doubling from tau, then Newton steps, bisection outside
+// the bracket.
+__device__ __forceinline__ float sr_bracket_f(float D, float m2, float S2, float B2, float tau, float g1)
+{
+    float Wlo = 0.0f, Whi = tau, f, df;
+    for (int k = 0; k < 64; ++k) {
+        if (sr_energy_f(Whi, D, m2, S2, B2, tau, g1, f, df) && f > 0.0f) break;
+        Wlo = Whi;
+        Whi *= 2.0f;
+    }
+    float W = Whi;
+    for (int it = 0; it < 50; ++it) {
+        float Wn = 0.5f * (W + Whi);
+        if (!sr_energy_f(W, D, m2, S2, B2, tau, g1, f, df)) {
+            Wlo = W;
+        } else {
+            if (f > 0.0f) Whi = W; else Wlo = W;
+            Wn = W - f / df;
+            if (!(Wn > Wlo && Wn < Whi)) Wn = 0.5f * (Wlo + Whi);
+            if (fabsf(Wn - W) <= 2.0e-6f * W) return Wn;
+        }
+        W = Wn;
+    }
+    return W;
+}
+
+// rho, v and p of a conserved state from the guess W0 (> 0, else tau - B^2/2)
+// for the ideal gas with g1 = (Gamma - 1) / Gamma.  ok: V holds the five
+// float32 values that sr_prim_mixed returns for the same state and guess
+// (rounded to float32), all of them physical.  Otherwise undecided.
+// Out of line: the sweeps recover three or four states a cell, and the copies
+// inlined (about 1000 instructions each) overflowed the instruction cache
+// (x sweep 36.1 ms at 256^3 with 15 of 20 stall cycles on instruction fetch).
+struct SrRec {
+    float V[5];
+    bool ok;
+};
+__device__ __forceinline__ bool sr_recover_in(const SrState &u, float W0, df g1, float (&V)[5])
+{
+    const df m2 = d_addp(d_addp(d_sqr(u.m[0]), d_sqr(u.m[1])), d_sqr(u.m[2]));
+    const df B2 = d_addp(d_addp(d_sqr(u.b[0]), d_sqr(u.b[1])), d_sqr(u.b[2]));
+    const df sx = d_mul(u.m[0], u.b[0]), sy = d_mul(u.m[1], u.b[1]), sz = d_mul(u.m[2], u.b[2]);
+    const df S = d_add(d_add(sx, sy), sz);
+    const float Sa = fabsf(sx.hi) + fabsf(sy.hi) + fabsf(sz.hi);
+    if (!(u.D.hi > 0.0f) || !(u.tau.hi > 0.0f)) return false;
+    if (!(W0 > 0.0f)) W0 = d_add(u.tau, d_neg(d_half(B2))).hi;
+    if (!(W0 > 0.0f)) return false;
+    // float32 Newton, as sr_prim_mixed; a two-cycle (the float32 residual's
+    // noise exceeds the criterion where B^2 >> W) runs to the same last
+    // iterate at once
+    const float S2f = d_sqr(S).hi;
+    float Wf = W0, Wp = 0.0f;
+    bool strict = false;
+    for (int it = 0; it < 12; ++it) {
+        float f, dfw;
+        strict = !sr_energy_f(Wf, u.D.hi, m2.hi, S2f, B2.hi, u.tau.hi, g1.hi, f, dfw);
+        const float Wn = Wf - f / dfw;
+        strict |= !(Wn > 0.0f);
+        if (strict) break;
+        if (Wn == Wp && fabsf(Wn - Wf) > 2.0e-6f * Wf) {
+            if (((11 - it) & 1) == 0) Wf = Wn;
+            break;
+        }
+        const bool done = fabsf(Wn - Wf) <= 2.0e-6f * Wf;
+        Wp = Wf;
+        Wf = Wn;
+        if (done) break;
+    }
+    // outside the physical range sr_prim_mixed hands over to the bracketed
+    // iteration, which converges to the root of the energy equation: so does
+    // this one, from a bracketed float32 iteration and with steps in
+    // double-float until one moves W by less than 2e-9
+    if (strict) Wf = sr_bracket_f(u.D.hi, m2.hi, S2f, B2.hi, u.tau.hi, g1.hi);
+    const float accept = strict ? 2.0e-9f : 1.0e-5f;
+    df W{Wf, 0.0f};
+#pragma unroll 1
+    for (int it = 0; it < 3; ++it) {
+        const df Wb = d_addp(W, B2), A = d_addp(W, Wb);
+        const df iW = d_rcp(W), iWb = d_rcp(Wb);
+        const df t = d_mul(S, iW), t2 = d_sqr(t);
+        const df iWb2 = d_sqr(iWb);
+        const df v2 = d_mul(d_addp(m2, d_mul(t2, A)), iWb2);
+        const df t2W = d_mul(t2, iW);
+        const df dv2 = d_mul(d_addp(v2, t2W), df{-2.0f * iWb.hi, -2.0f * iWb.lo});
+        const df ev = d_addf(d_neg(v2), 1.0f);
+        if (!(ev.hi > 0.0f)) return false;
+        const df is = d_rsqrt(ev);
+        const df Ds = d_mul(u.D, d_mul(ev, is));
+        const df p = d_mul(g1, d_add(d_mul(W, ev), d_neg(Ds)));
+        const df dp = d_mul(g1, d_add(ev, d_mul(dv2, d_add(d_half(d_mul(u.D, is)), d_neg(W)))));
+        const df hB = d_half(B2);
+        // f = W - p + B^2 (1 + v^2)/2 - t^2/2 - tau
+        const df f = d_add(d_add(d_add(d_add(W, d_neg(u.tau)), hB), d_mul(hB, v2)), d_neg(d_add(p, d_half(t2))));
+        const df dF = d_addf(d_add(d_add(d_neg(dp), d_mul(hB, dv2)), t2W), 1.0f);
+        const df dW = d_neg(d_mul(f, d_rcp(dF)));
+        const df Wn = d_add(W, dW);
+        if (!(Wn.hi > 0.0f)) return false;
+        const float a = fabsf(dW.hi), lim = accept * W.hi;
+        if (a > 0.9999f * lim) {
+            if (!(a > 1.0001f * lim)) return false;
+            W = Wn;
+            continue;
+        }
+        const df evn = d_add(ev, d_neg(d_mul(dv2, dW)));
+        const df pn = d_add(p, d_mul(dp, dW));
+        if (!(evn.hi > 0.0f)) return false;
+        const df iWbn = d_rcp(d_addp(Wn, B2)), SW = d_mul(S, d_rcp(Wn));
+        const df rho = d_mul(u.D, d_mul(evn, d_rsqrt(evn)));
+        if (!(rho.hi > 0.0f) || !(pn.hi > 0.0f)) return false;
+        // error bounds (absolute), see SR_MARGIN
+        const float Ta = Sa * iW.hi, v2b = (m2.hi + Ta * Ta * A.hi) * iWb2.hi;
+        const float e_ev = SR_K_EV * v2b, Dis = u.D.hi * is.hi;
+        const float e_p0 = g1.hi * ((W.hi + 0.5f * Dis) * e_ev + 2.0f * SR_K_F * Ds.hi);
+        const float e_f = e_p0 + hB.hi * e_ev + SR_K_F * (W.hi + B2.hi + 0.5f * Ta * Ta + u.tau.hi);
+        const float e_W = e_f / fabsf(dF.hi);
+        const float e_evn = e_ev + fabsf(dv2.hi) * e_W;
+        const bool sure =
+            d_certain(pn, SR_MARGIN * (e_p0 + fabsf(dp.hi) * e_W)) &&
+            d_certain(rho, SR_MARGIN * (0.5f * Dis * e_evn + SR_K_V * rho.hi));
+        if (!sure) return false;
+        V[0] = rho.hi;
+        V[4] = pn.hi;
+        // low parts lost below the float range: 2^-98 absolute in each m_k
+        const float tiny = 3.2e-30f, bs = (fabsf(u.b[0].hi) + fabsf(u.b[1].hi) + fabsf(u.b[2].hi)) * iW.hi;
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const df sb = d_mul(SW, u.b[k]);
+            const df v = d_mul(d_add(u.m[k], sb), iWbn);
+            const float bi = fabsf(u.b[k].hi);
+            const float e_v = SR_K_V * (fabsf(u.m[k].hi) + Ta * bi) + (fabsf(v.hi) + fabsf(SW.hi) * bi * iW.hi) * e_W;
+            const bool zero = u.m[k].hi == 0.0f && sb.hi == 0.0f && u.m[k].lo == 0.0f && sb.lo == 0.0f && Ta * bi == 0.0f;
+            ok &= zero || d_certain(v, iWbn.hi * (SR_MARGIN * e_v + tiny * (1.0f + bi * bs)));
+            V[1 + k] = v.hi;
+        }
+        return ok;
+    }
+    return false;
+}
+
+static __device__ __noinline__ SrRec sr_recover_call(SrState u, float W0, df g1)
+{
+    SrRec r;
+    r.ok = sr_recover_in(u, W0, g1, r.V);
+    return r;
+}
+__device__ __forceinline__ bool sr_recover(const SrState &u, float W0, df g1, float (&V)[5])
+{
+    const SrRec r = sr_recover_call(u, W0, g1);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) V[q] = r.V[q];
+    return r.ok;
+}
+
+// ---- the float64 iteration for the lanes sr_recover leaves undecided; out of
+// line where its registers and code can stay off the fast path
+
+struct SrCons {
+    double U[NV];
+};
+struct SrFace {
+    float V[NV], T[NV];
+};
+struct SrOut {
+    float V[NV];
+    unsigned int st;
+};
+
+static __device__ __noinline__ SrOut sr_prim_slow(SrCons c, double gam, double W0)
+{
+    double V[NV];
+    SrOut o;
+    o.st = sr_prim_mixed(c.U, gam, V, W0);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) o.V[q] = (float)V[q];
+    return o;
+}
+
+static __device__ __noinline__ SrOut sr_interface_slow(SrFace f, double gam)
+{
+    double V[NV];
+    SrOut o;
+    o.st = sr_interface64<float>(f.V, f.T, gam, V);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) o.V[q] = (float)V[q];
+    return o;
+}
+
+// f.V: the cell's V^n, f.T: the increment x (sr_mh_recover)
+__device__ __forceinline__ SrOut sr_mh_slow(SrCons c, SrFace f, double gam)
+{
+    double V[NV];
+    SrOut o;
+    o.st = sr_mh_recover<float>(c.U, f.V, f.T, gam, V);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) o.V[q] = (float)V[q];
+    return o;
+}
+
+// Interface state of the mixed path, V(U(f.V) + f.T): the double-float recovery
+// (ideal gas), else the float64 one.  Out of line, as sr_recover: each sweep
+// needs it twice a cell.
+static __device__ __noinline__ SrOut sr_interface_call(SrFace f, df g1, df ig1, double gam)
+{
+    if (g1.hi > 0.0f) {
+        SrState u;
+        float W0, v[5];
+        sr_state_of(f.V, f.T, ig1, u, W0);
+        if (sr_recover(u, W0, g1, v)) {
+            SrOut o;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) o.V[q] = v[q];
+#pragma unroll
+            for (int q = 5; q < NV; ++q) o.V[q] = __fadd_rn(f.V[q], f.T[q]);
+            o.st = 0u;
+            return o;
+        }
+    }
+    return sr_interface_slow(f, gam);
+}
+
+// A float64 value as a normalised double-float.
+__device__ __forceinline__ df sr_split(double x)
+{
+    const df s = df_split(x);
+    return d_norm(s.hi, s.lo);
+}
+
+// sr_mh_predict of the mixed path (global component gp(q) of the pool at Uc[
+// gp(q) us] is local component q): U* = U_i^n - x in double-float, recovered by
+// sr_recover.  B and psi of the half-step state are U*'s, rounded; where
+// double-float leaves one undecided the float64 path takes the cell.
+template <class GP>
+__device__ __forceinline__ unsigned int sr_mh_predict_f(const float (&vm1)[NV], const float (&v0)[NV],
+                                                        const float (&vp1)[NV], const double *Uc, long long us, GP gp,
+                                                        float gam, float ch, float dtdx, double gamd, df g1, df ig1,
+                                                        float (&Vp)[NV], float (&Vm)[NV])
+{
+    float dV[NV], x[NV], V[NV];
+    sr_mh_increment<float>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+    unsigned int st = 0;
+    bool ok = false;
+    if (g1.hi > 0.0f) {
+        SrState u;
+        df d[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) d[q] = d_addf(sr_split(Uc[gp(q) * us]), -x[q]);
+        u.D = d[0];
+        u.tau = d_add(d[4], d[0]);
+        ok = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            u.m[k] = d[1 + k];
+            u.b[k] = d[5 + k];
+        }
+#pragma unroll
+        for (int q = 5; q < NV; ++q) {
+            V[q] = d[q].hi;
+            ok &= d_certain(d[q], 4.0f * SR_MARGIN * (fabsf(d[q].hi) + 2.0f * fabsf(x[q])) + 1.0e-37f) ||
+                  (d[q].hi == 0.0f && x[q] == 0.0f);
+        }
+        df ev, W;
+        sr_w_of(v0, ig1, ev, W);
+        float v[5];
+        ok = ok && sr_recover(u, W.hi, g1, v);
+#pragma unroll
+        for (int q = 0; q < 5; ++q) V[q] = v[q];
+    }
+    if (!ok) {
+        SrCons c;
+        SrFace f;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            c.U[q] = Uc[gp(q) * us];
+            f.V[q] = v0[q];
+            f.T[q] = x[q];
+        }
+        const SrOut o = sr_mh_slow(c, f, gamd);
+        st = o.st;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) V[q] = o.V[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        Vp[q] = V[q] + 0.5f * dV[q];
+        Vm[q] = V[q] - 0.5f * dV[q];
+    }
+    return st;
+}
+
+} // namespace ctu

@@ -409,16 +409,14 @@ __device__ __forceinline__ void riemann_hll_sr(const R (&L0)[NV], const R (&R0)[
     F[8] = ch * ch * Bm;
 }
 
-// MUSCL-Hancock normal predictor of one cell (Section 3.3, beta = 1):
-// vs = V_(i-1), V_i, V_(i+1) (local order, precision R), U0 = U_i^n (local,
-// float64).  U* = U0 - dt/(2 dx) [F(V_+) - F(V_-)] and its recovery in
-// float64; V*_(+/-) = V(U*) +/- dV/2.
+// The slopes and the flux increment of the MUSCL-Hancock normal predictor
+// (Section 3.3, beta = 1): vs = V_(i-1), V_i, V_(i+1) (local order), x =
+// dt/(2 dx) [F(V_+) - F(V_-)] with V_(+/-) = V_i +/- dV/2.
 template <class R>
-__device__ __forceinline__ unsigned int sr_mh_predict(const R (&vm1)[NV], const R (&v0)[NV], const R (&vp1)[NV],
-                                                      const double (&U0)[NV], R gam, R ch, R dtdx, double gamd,
-                                                      R (&Vp)[NV], R (&Vm)[NV])
+__device__ __forceinline__ void sr_mh_increment(const R (&vm1)[NV], const R (&v0)[NV], const R (&vp1)[NV], R gam, R ch,
+                                                R dtdx, R (&dV)[NV], R (&x)[NV])
 {
-    R dV[NV], Vpl[NV], Vmi[NV];
+    R Vpl[NV], Vmi[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
         dV[q] = mc_slope(v0[q] - vm1[q], vp1[q] - v0[q]);
@@ -430,20 +428,56 @@ __device__ __forceinline__ unsigned int sr_mh_predict(const R (&vm1)[NV], const 
     sr_cons<R, R>(Vmi, gam, Um);
     sr_flux(Vpl, Up, gam, ch, Fp);
     sr_flux(Vmi, Um, gam, ch, Fm);
-    double Us[NV], Vs[NV];
     const R h = R(0.5) * dtdx;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) Us[q] = U0[q] - (double)(h * (Fp[q] - Fm[q]));
-    // Newton starts from the cell-centre W = w gamma^2 (U* is an O(dt) update of U_i)
+    for (int q = 0; q < NV; ++q) x[q] = h * (Fp[q] - Fm[q]);
+}
+
+// The half-step state V(U*), U* = U_i^n - x, in float64.  Newton starts from
+// the cell-centre W = w gamma^2 (U* is an O(dt) update of U_i).
+template <class R>
+__device__ __forceinline__ unsigned int sr_mh_recover(const double (&U0)[NV], const R (&v0)[NV], const R (&x)[NV],
+                                                      double gamd, double (&Vs)[NV])
+{
+    double Us[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) Us[q] = U0[q] - (double)x[q];
     const double v2c = (double)v0[1] * v0[1] + (double)v0[2] * v0[2] + (double)v0[3] * v0[3];
     const double Wc = sr_w<double>((double)v0[0], (double)v0[4], gamd) * rcp64(1.0 - v2c);
-    const unsigned int st = sr_prim<R>(Us, gamd, Vs, Wc);
+    return sr_prim<R>(Us, gamd, Vs, Wc);
+}
+
+// MUSCL-Hancock normal predictor of one cell: V*_(+/-) = V(U*) +/- dV/2,
+// U0 = U_i^n (local, float64).
+template <class R>
+__device__ __forceinline__ unsigned int sr_mh_predict(const R (&vm1)[NV], const R (&v0)[NV], const R (&vp1)[NV],
+                                                      const double (&U0)[NV], R gam, R ch, R dtdx, double gamd,
+                                                      R (&Vp)[NV], R (&Vm)[NV])
+{
+    R dV[NV], x[NV];
+    sr_mh_increment<R>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+    double Vs[NV];
+    const unsigned int st = sr_mh_recover<R>(U0, v0, x, gamd, Vs);
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
         Vp[q] = (R)Vs[q] + R(0.5) * dV[q];
         Vm[q] = (R)Vs[q] - R(0.5) * dV[q];
     }
     return st;
+}
+
+// Interface state at n+1/2 in float64: V(U(W) + T), Newton from the W of the
+// predicted state (the transverse correction T is an O(dt) change).
+template <class R>
+__device__ __forceinline__ unsigned int sr_interface64(const R (&W)[NV], const R (&T)[NV], double gamd, double (&V)[NV])
+{
+    double U[NV];
+    sr_cons<double, R>(W, gamd, U);
+    const double v2 = (double)W[1] * W[1] + (double)W[2] * W[2] + (double)W[3] * W[3];
+    const double W0 = sr_w<double>((double)W[0], (double)W[4], gamd) * rcp64(1.0 - v2);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) U[q] += (double)T[q];
+    return sr_prim<R>(U, gamd, V, W0);
 }
 
 } // namespace ctu

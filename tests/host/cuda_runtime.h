@@ -1,0 +1,33 @@
+// Host stand-ins for the CUDA names the relativistic recovery's headers use, so
+// that its arithmetic can be compiled and checked by the host compiler.
+#pragma once
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#define __device__
+#define __host__
+#define __forceinline__ inline
+#define __noinline__
+using std::fabs;
+using std::fmax;
+using std::fmin;
+using std::isfinite;
+inline float __fadd_rn(float a, float b) { return a + b; }
+inline float __fmul_rn(float a, float b) { return a * b; }
+inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
+inline float __fdividef(float a, float b) { return a / b; }
+inline float rsqrtf(float x) { return (float)(1.0 / std::sqrt((double)x)); }
+template <class T, class F> inline T bits_as(F f)
+{
+    T t;
+    static_assert(sizeof(T) == sizeof(F), "same size");
+    std::memcpy(&t, &f, sizeof(T));
+    return t;
+}
+inline int __double2hiint(double x) { return (int)(bits_as<uint64_t>(x) >> 32); }
+inline int __double2loint(double x) { return (int)(uint32_t)bits_as<uint64_t>(x); }
+inline double __hiloint2double(int h, int l) { return bits_as<double>(((uint64_t)(uint32_t)h << 32) | (uint32_t)l); }
+inline float __uint_as_float(unsigned u) { return bits_as<float>(u); }
+inline unsigned __float_as_uint(float f) { return bits_as<unsigned>(f); }
+inline long long __double_as_longlong(double d) { return bits_as<long long>(d); }
+inline double __longlong_as_double(long long u) { return bits_as<double>(u); }
