@@ -390,7 +390,7 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
 /* The tile width *xw and segment length *seg the context uses for patches of
  * interior shape n[3] (autotuned if ctu_autotune saw that shape, else the
  * default rule: 32 lanes for n[0] >= 24, 16 for n[0] >= 12, else 8; 16
- * cells). */
+ * cells, which a step replaces by the length that suits the whole batch). */
 ctu_status ctu_tile_params(ctu_ctx *ctx, const int n[3], int *xw, int *seg);
 
 /* ---- Level operators (Section 4 of Mignone et al. 2012; Cartesian) ------

@@ -99,8 +99,8 @@ static bool grid_fits(const std::vector<Group> &gs, int ndim)
         tot[0] += c * Tiles::ghosted(G.N);
         for (int D = 0; D < 3; ++D) {
             // (one row per thread: the most blocks the x kernels launch)
-            tot[1 + D] += c * Tiles::div1(G.n, ndim, D, G.xw, G.seg, true, 1);
-            tot[4 + D] += c * (D == 0 ? Tiles::sweep_x(G.n, G.xw, 1) : Tiles::sweep_m(G.n, D, G.xw, G.seg));
+            tot[1 + D] += c * Tiles::div1(G.n, ndim, D, D == 0 ? G.dx : G.rw, G.seg, true, 1);
+            tot[4 + D] += c * (D == 0 ? Tiles::sweep_x(G.n, G.sx, 1) : Tiles::sweep_m(G.n, D, G.xw, G.seg));
         }
         tot[7] += c * Tiles::interior(G.n, G.xw);
     }
@@ -313,8 +313,14 @@ static ctu_status bind_patches(ctu_ctx *ctx, const ctu_patch *p, int np, cudaStr
         const auto it = ctx->tune.find(shape_key(G.n));
         G.xw = it != ctx->tune.end() ? it->second[0] : Tiles::xw(G.n[0]);
         G.seg = it != ctx->tune.end() ? it->second[1] : SEG;
+        group_widths(G, ctx->cfg.ndim, ctx->cfg.precision == CTU_FP64, ctx->cfg.corner == CTU_CORNER_MT);
     }
     if (!grid_fits(g2, ctx->cfg.ndim)) return CTU_EINVAL;
+    std::vector<Group> g3(g2);
+    choose_segments(g3.data(), (int)g3.size(), ctx->cfg.ndim, ctx->cfg.precision == CTU_FP64,
+                    ctx->cfg.physics == CTU_SRMHD, ctx->sms,
+                    [&](const Group &G) { return ctx->tune.find(shape_key(G.n)) == ctx->tune.end(); });
+    if (grid_fits(g3, ctx->cfg.ndim)) g2.swap(g3);
     if (np > ctx->dpatch_cap) {
         if (ctx->dpatch) cudaFree(ctx->dpatch);
         ctx->dpatch = nullptr;

@@ -188,6 +188,8 @@ struct GroupTable {
     int xw[MAXG];
     int seg[MAXG];
     unsigned char xr[MAXG];  // rows per thread of the x-tiled kernels that take several (rows_per_thread)
+    // row widths (lanes): x sweep, first-order x stage, marching first-order kernels
+    int sx[MAXG], dx[MAXG], rw[MAXG];
 };
 
 // Division of 0 <= x < 2^32 by an invariant divisor d >= 1 with one high
@@ -211,7 +213,7 @@ inline DivMagic divmagic(unsigned d)
 }
 
 struct Where {
-    int patch, b, xw, seg, xr;
+    int patch, b, xw, seg, xr, sx, dx, rw;
 };
 
 __device__ __forceinline__ Where locate(const GroupTable &gt)
@@ -229,6 +231,9 @@ __device__ __forceinline__ Where locate(const GroupTable &gt)
     w.xw = gt.xw[g];
     w.seg = gt.seg[g];
     w.xr = gt.xr[g];
+    w.sx = gt.sx[g];
+    w.dx = gt.dx[g];
+    w.rw = gt.rw[g];
     return w;
 }
 // The marching sweeps are latency bound: they are compiled for at least
@@ -260,23 +265,63 @@ __host__ __device__ __forceinline__ int tile_xw(int nx)
     return nx >= 24 ? 32 : (nx >= 12 ? 16 : 8);
 }
 
-// Row width of the x sweep's tile: a patch row of up to 32 cells takes one
-// row of n_x + 2 lanes (its traced cells, the rows packed BLOCK / (n_x + 2)
-// to a block), so that small patches leave few lanes idle; wider rows take
-// the group's width w (8, 16 or 32).  The exchange between the lanes of a row
-// goes through shared memory, so a row need not be a power of two wide.
-__host__ __device__ __forceinline__ int sweepx_xw(int nx, int w)
+// Row widths of the x-tiled kernels, chosen on the host per patch shape: a
+// row of n_x cells is cut into tiles of w lanes, of which w - halo yield a
+// cell, and a block takes BLOCK / w rows, so the lanes left idle at the halo,
+// at the last tile and beyond the last full row depend on how w divides n_x.
+// The width with the fewest blocks for `rows` rows wins (the widest on a tie:
+// fewer tiles, longer contiguous loads).  With 32 lanes throughout a 64^3
+// patch ran three tiles for its 66 traced cells (67% of the lanes yielding a
+// cell), now four of 18 lanes (87%); 96^3 in float64: x sweep 3.94 -> 3.47 ms.
+// Longer than 34 lanes (32 cells and the halo) no width gains.
+inline int tile_blocks(int cells, int rows, int w, int halo)
 {
-    return nx <= 32 ? nx + 2 : w;
+    const int per = BLOCK / w;
+    return ((cells + w - halo - 1) / (w - halo)) * ((rows + per - 1) / per);
 }
-
-// Row width of the marching first-order kernels (k_div1 and k_pred along y
-// and z), whose lanes cover x in [-1, n_x]: the same packing, n_x + 2 lanes
-// per row for rows of up to 32 cells (the lanes of a row do not exchange
-// values, so any width serves).
-__host__ __device__ __forceinline__ int ringx_xw(int nx, int w)
+// x sweep (halo 2): its lanes exchange through shared memory, any width
+// serves.  In float32 a tenth fewer blocks at least: narrow rows read partial
+// sectors (128^3: 18 lanes, 9% fewer blocks, 264 us against 262); float64 is bound
+// by its pipe (2-D 128^2: 18 lanes, 5% fewer blocks, 61 us against 105).
+inline int sweepx_width(const int *n, bool f64)
 {
-    return nx <= 32 ? nx + 2 : w;
+    const int w0 = n[0] <= 32 ? n[0] + 2 : 32;
+    int best = w0;
+    for (int w = 34; w >= 6; --w)
+        if (w - 2 <= n[0] && tile_blocks(n[0], n[1], w, 2) < tile_blocks(n[0], n[1], best, 2)) best = w;
+    return f64 || 10 * tile_blocks(n[0], n[1], best, 2) <= 9 * tile_blocks(n[0], n[1], w0, 2) ? best : w0;
+}
+// First-order x stage (halo 1): the lanes exchange by warp shuffles, a power
+// of two.
+inline int div1x_width(const int *n, int ndim)
+{
+    const int rows = ndim > 1 ? n[1] + 2 : 1;
+    int best = 32;
+    for (int w = 16; w >= 8; w /= 2)
+        if (tile_blocks(n[0], rows, w, 1) < tile_blocks(n[0], rows, best, 1)) best = w;
+    return best;
+}
+// Marching first-order kernels (k_div1, k_pred along y, z), whose lanes cover
+// x in [-1, n_x] and exchange nothing: the width that leaves the fewest lanes
+// idle, less `pen` for every lane short of 32 (each row of a warp starts a
+// memory sector of its own): 0.01 for k_div1 in float32 (256^3, where every
+// width is full: 16 lanes 1.11 ms against 0.98), 0.004 for k_pred, which does four
+// times the work on the same data (128^3: 8 lanes 441 us, 32 lanes 471), 0 in
+// float64, bound by its pipe (2-D 128^2: 8 lanes 70 us, 32 lanes 103).
+inline int ring_width(const int *n, double pen)
+{
+    const int cells = n[0] + 2;
+    int best = 0;
+    double top = 0.0;
+    for (int w = cells < 34 ? cells : 34; w > 0 && (best == 0 || w >= 8); --w) {
+        const double use = (double)cells * (BLOCK / w) / ((cells + w - 1) / w * BLOCK);
+        const double v = use * (w < 32 ? 1.0 - pen * (32 - w) : 1.0);
+        if (v > top) {
+            top = v;
+            best = w;
+        }
+    }
+    return best;
 }
 
 // k_prim's trimmed box (see k_prim) serves patches whose ghosted rows are at
@@ -871,17 +916,18 @@ struct Tiles {
         return ((long long)(N[0] - 2) * (N[1] > 1 ? N[1] - 2 : 1) * (N[2] > 1 ? N[2] - 2 : 1) + BLOCK * PRIM_CELLS - 1) /
                (BLOCK * PRIM_CELLS);
     }
-    // ext: along D also the ring's layers -1 and n_D (k_div1's EXT)
     // rows per thread of k_div1<0> and of k_sweep_x on patches of n cells,
-    // at most `most`
+    // at most `most` (w: their row widths, div1x_width and sweepx_width)
     static int div1x_rows(const int *n, int ndim, int w, int most)
     {
         return rows_per_thread(most, ndim > 1 ? n[1] + 2 : 1, BLOCK / w);
     }
     static int sweepx_rows(const int *n, int w, int most)
     {
-        return rows_per_thread(most, n[1], BLOCK / sweepx_xw(n[0], w));
+        return rows_per_thread(most, n[1], BLOCK / w);
     }
+    // w: div1x_width for D = 0, ring_width else; ext: along D also the ring's
+    // layers -1 and n_D (k_div1's EXT)
     static long long div1(const int *n, int ndim, int D, int w, int seg, bool ext = false, int most = DIV1X_ROWS)
     {
         const int r = BLOCK / w;
@@ -894,8 +940,7 @@ struct Tiles {
         const int O = D == 1 ? 2 : 1;
         const int eO = ndim > O ? n[O] + 2 : 1;
         const long long nseg = (n[D] + x2 + seg - 1) / seg;
-        const int wr = ringx_xw(n[0], w), rr = BLOCK / wr;
-        return (long long)((n[0] + 2 + wr - 1) / wr) * ((eO * nseg + rr - 1) / rr);
+        return (long long)((n[0] + 2 + w - 1) / w) * ((eO * nseg + r - 1) / r);
     }
     // the corner coupling's transverse fluxes along x (k_pred<0>): traced
     // cells [-1, n_x], rows and planes over the ring [-1, n]
@@ -907,9 +952,7 @@ struct Tiles {
     }
     static long long sweep_x(const int *n, int w, int most = SWEEPX_ROWS)
     {
-        const int xr = sweepx_rows(n, w, most);
-        w = sweepx_xw(n[0], w);
-        const int rr = (BLOCK / w) * xr;  // rows of a block
+        const int rr = (BLOCK / w) * sweepx_rows(n, w, most);  // rows of a block
         return (long long)((n[0] + w - 3) / (w - 2)) * ((n[1] + rr - 1) / rr) * n[2];
     }
     static long long sweep_m(const int *n, int D, int w, int seg)
@@ -1112,7 +1155,7 @@ __global__ void __launch_bounds__(BLOCK) k_div1(StepArgs a, GroupTable gt, const
 {
     const Where wh = locate(gt);
     const DevPatch P = a.patches[wh.patch];
-    const Tile t(D == 0 ? wh.xw : ringx_xw(P.n[0], wh.xw));
+    const Tile t(D == 0 ? wh.dx : wh.rw);
     const int SEGL = wh.seg;
     const R gam = pgam<R>(a), ch = pch<R>(a.sp);
     const R iD = pidx<R>(P, D);
@@ -1236,7 +1279,7 @@ __global__ void __launch_bounds__(BLOCK) k_pred(StepArgs a, GroupTable gt, const
 {
     const Where wh = locate(gt);
     const DevPatch P = a.patches[wh.patch];
-    const Tile t(D == 0 ? wh.xw : ringx_xw(P.n[0], wh.xw));
+    const Tile t(D == 0 ? wh.xw : wh.rw);
     const R gam = pgam<R>(a), ch = pch<R>(a.sp);
     const R dtr = pdt<R>(a.sp);
     const R iD = pidx<R>(P, D);
@@ -1346,7 +1389,7 @@ __global__ void __launch_bounds__(BLOCK, sizeof(R) == 4 ? (recon_par(PPM) ? CTU_
     const Where wh = locate(gt);
     const int patch = wh.patch;
     const DevPatch P = a.patches[patch];
-    const Tile t(sweepx_xw(P.n[0], wh.xw));
+    const Tile t(wh.sx);
     const int out_x = t.xw - 2;
     const int xr = wh.xr;         // rows of a thread (Tiles::sweepx_rows)
     const int RR = t.rows * xr;  // rows of a block

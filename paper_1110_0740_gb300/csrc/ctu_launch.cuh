@@ -41,6 +41,9 @@ static int over_groups(const LaunchInfo &li, BPP bpp, GO go, XR xr = XR())
             gt.xw[k] = G.xw;
             gt.seg[k] = G.seg;
             gt.xr[k] = (unsigned char)xr(G);
+            gt.sx[k] = G.sx;
+            gt.dx[k] = G.dx;
+            gt.rw[k] = G.rw;
             tot += (long long)G.count * gt.bpp[k];
         }
         gt.start[gt.n] = (int)tot;
@@ -170,11 +173,11 @@ static int launch_step_t(const StepArgs &a, const LaunchInfo &li, cudaStream_t s
                 li, [&](const Group &G) { return Tiles::pred_x(G.n, a.ndim, G.xw); },
                 [&](const GroupTable &gt, unsigned nb) { k_pred<PHYS, R, PPM, 0><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.xw, G.seg); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg); },
                 [&](const GroupTable &gt, unsigned nb) { k_pred<PHYS, R, PPM, 1><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
             if (a.ndim > 2)
                 n += over_groups(
-                    li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.xw, G.seg); },
+                    li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg); },
                     [&](const GroupTable &gt, unsigned nb) {
                         k_pred<PHYS, R, PPM, 2><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1);
                     });
@@ -183,19 +186,19 @@ static int launch_step_t(const StepArgs &a, const LaunchInfo &li, cudaStream_t s
     } else if (a.ndim > 1 || EXT) {
         CTU_MARK("flux1");
         const int xr1 = launch_rows(li, DIV1X_ROWS, [&](const Group &G, int x) {
-            return Tiles::div1(G.n, a.ndim, 0, G.xw, G.seg, EXT, x);
+            return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg, EXT, x);
         });
         n += over_groups(
-            li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 0, G.xw, G.seg, EXT, xr1); },
+            li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg, EXT, xr1); },
             [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 0, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); },
-            [&](const Group &G) { return Tiles::div1x_rows(G.n, a.ndim, G.xw, xr1); });
+            [&](const Group &G) { return Tiles::div1x_rows(G.n, a.ndim, G.dx, xr1); });
         if (a.ndim > 1)
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.xw, G.seg, EXT); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg, EXT); },
                 [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 1, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
         if (a.ndim > 2)
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.xw, G.seg, EXT); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg, EXT); },
                 [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 2, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
         CTU_MARK(nullptr);
     }
@@ -257,13 +260,13 @@ static int launch_step_t(const StepArgs &a, const LaunchInfo &li, cudaStream_t s
         CTU_MARK(nullptr);
     }
     CTU_MARK("sweep_x");
-    const int xrs = launch_rows(li, SWEEPX_ROWS, [&](const Group &G, int x) { return Tiles::sweep_x(G.n, G.xw, x); });
+    const int xrs = launch_rows(li, SWEEPX_ROWS, [&](const Group &G, int x) { return Tiles::sweep_x(G.n, G.sx, x); });
     n += over_groups(
-        li, [&](const Group &G) { return Tiles::sweep_x(G.n, G.xw, xrs); },
+        li, [&](const Group &G) { return Tiles::sweep_x(G.n, G.sx, xrs); },
         [&](const GroupTable &gt, unsigned nb) {
             k_sweep_x<PHYS, R, PPM, IF64, 1><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1, A);
         },
-        [&](const Group &G) { return Tiles::sweepx_rows(G.n, G.xw, xrs); });
+        [&](const Group &G) { return Tiles::sweepx_rows(G.n, G.sx, xrs); });
     CTU_MARK(nullptr);
     return n;
 }

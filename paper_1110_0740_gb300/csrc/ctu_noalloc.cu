@@ -130,6 +130,7 @@ extern "C" ctu_status ctu_step_noalloc(const ctu_config *cfg, const double *U_in
         }
         groups[i].xw = Tiles::xw(q.n[0]);
         groups[i].seg = SEG;
+        group_widths(groups[i], cfg->ndim, cfg->precision == CTU_FP64, false);
     }
     const size_t elt = cfg->precision == CTU_FP64 ? sizeof(double) : sizeof(float);
     if ((size_t)off * SCRATCH_ARRAYS * elt > kScratchBytes) return CTU_ETOOLARGE;
@@ -201,6 +202,8 @@ extern "C" ctu_status ctu_step_noalloc(const ctu_config *cfg, const double *U_in
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
             li.sms = sms;
     }
+    choose_segments(groups, npatch, cfg->ndim, cfg->precision == CTU_FP64, false, li.sms,
+                    [](const Group &) { return true; });
     if (cfg->precision == CTU_FP64)
         launch_step<double>(a, li, s);
     else
