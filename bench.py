@@ -1055,7 +1055,7 @@ def precision_split_roofline(n, cells_per_s, hbm_gbs):
             "frac": cells_per_s / bounds[binding]}
 
 
-STEP_SOURCES = ("df.cuh", "mhd_device.cuh", "srmhd_device.cuh", "sr_df.cuh", "ctu_kernels.cuh", "ctu_launch.h",
+STEP_SOURCES = ("df.cuh", "mhd_device.cuh", "mhd_fp64.cuh", "srmhd_device.cuh", "sr_df.cuh", "ctu_kernels.cuh", "ctu_launch.h",
                 "ctu_launch.cuh", "par_ops.cuh", "ctu_f32.cu", "_build.py")
 
 

@@ -99,7 +99,7 @@ static bool grid_fits(const std::vector<Group> &gs, int ndim)
         tot[0] += c * Tiles::ghosted(G.N);
         for (int D = 0; D < 3; ++D) {
             // (one row per thread: the most blocks the x kernels launch)
-            tot[1 + D] += c * Tiles::div1(G.n, ndim, D, D == 0 ? G.dx : G.rw, G.seg, true, 1);
+            tot[1 + D] += c * Tiles::div1(G.n, ndim, D, D == 0 ? G.dx : G.rw, G.seg1, true, 1);
             tot[4 + D] += c * (D == 0 ? Tiles::sweep_x(G.n, G.sx, 1) : Tiles::sweep_m(G.n, D, G.xw, G.seg));
         }
         tot[7] += c * Tiles::interior(G.n, G.xw);
@@ -313,6 +313,7 @@ static ctu_status bind_patches(ctu_ctx *ctx, const ctu_patch *p, int np, cudaStr
         const auto it = ctx->tune.find(shape_key(G.n));
         G.xw = it != ctx->tune.end() ? it->second[0] : Tiles::xw(G.n[0]);
         G.seg = it != ctx->tune.end() ? it->second[1] : SEG;
+        G.seg1 = SEG;
         group_widths(G, ctx->cfg.ndim, ctx->cfg.precision == CTU_FP64, ctx->cfg.corner == CTU_CORNER_MT);
     }
     if (!grid_fits(g2, ctx->cfg.ndim)) return CTU_EINVAL;
@@ -397,6 +398,7 @@ static StepArgs make_args(const ctu_ctx *ctx, const double *Uin, double *Uout, i
     a.gm1f = tm ? 0.0f : (float)(ctx->cfg.gamma - 1.0);
     if (ctx->cfg.physics == CTU_SRMHD && !tm) {
         const double ig = ctx->cfg.gamma / (ctx->cfg.gamma - 1.0), g1 = (ctx->cfg.gamma - 1.0) / ctx->cfg.gamma;
+        a.sr_g1 = g1;
         a.sr_g1h = (float)g1;
         a.sr_g1l = (float)(g1 - (double)a.sr_g1h);
         a.sr_igh = (float)ig;

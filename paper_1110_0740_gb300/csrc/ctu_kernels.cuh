@@ -31,6 +31,7 @@
 
 #include "df.cuh"
 #include "mhd_device.cuh"
+#include "mhd_fp64.cuh"
 #include "srmhd_device.cuh"
 #include "sr_df.cuh"
 
@@ -73,6 +74,7 @@ struct StepArgs {
     // relativistic ideal gas: (Gamma-1)/Gamma and its inverse as double-float
     // pairs (0 with the Taub-Mathews equation of state)
     float sr_g1h, sr_g1l, sr_igh, sr_igl;
+    double sr_g1;          // (Gamma-1)/Gamma
     double glm_alpha;
     int upwind;            // tracing mode (CTU_TRACE_*); 2 and 3 only in the reference-state kernels
     int limiter;           // linear reconstruction's slope (CTU_LINEAR_*), RECON_LIN kernels
@@ -186,7 +188,7 @@ struct GroupTable {
     unsigned bm[MAXG];       // division by bpp: multiplier and shifts (divmagic)
     unsigned char bs1[MAXG], bs2[MAXG];
     int xw[MAXG];
-    int seg[MAXG];
+    int seg[MAXG], seg1[MAXG];  // marching segment of the sweeps, of the first-order kernels
     unsigned char xr[MAXG];  // rows per thread of the x-tiled kernels that take several (rows_per_thread)
     // row widths (lanes): x sweep, first-order x stage, marching first-order kernels
     int sx[MAXG], dx[MAXG], rw[MAXG];
@@ -213,7 +215,7 @@ inline DivMagic divmagic(unsigned d)
 }
 
 struct Where {
-    int patch, b, xw, seg, xr, sx, dx, rw;
+    int patch, b, xw, seg, seg1, xr, sx, dx, rw;
 };
 
 __device__ __forceinline__ Where locate(const GroupTable &gt)
@@ -230,6 +232,7 @@ __device__ __forceinline__ Where locate(const GroupTable &gt)
     w.b = (int)rel - q * gt.bpp[g];
     w.xw = gt.xw[g];
     w.seg = gt.seg[g];
+    w.seg1 = gt.seg1[g];
     w.xr = gt.xr[g];
     w.sx = gt.sx[g];
     w.dx = gt.dx[g];
@@ -405,7 +408,13 @@ template <class R> __device__ __forceinline__ unsigned int prim_of(const double 
 template <>
 __device__ __forceinline__ unsigned int prim_of<double>(const double (&U)[NV], const StepArgs &a, double (&V)[NV])
 {
-    return prim_from_cons64(U, a.gam - 1.0, V) ? 0u : state_flags(V[0], V[4]);
+    const double ir = d_rcp64(U[0]);
+    const double vx = U[1] * ir, vy = U[2] * ir, vz = U[3] * ir;
+    const double ke = U[1] * vx + U[2] * vy + U[3] * vz;
+    const double me = U[5] * U[5] + U[6] * U[6] + U[7] * U[7];
+    V[0] = U[0]; V[1] = vx; V[2] = vy; V[3] = vz; V[4] = (a.gam - 1.0) * fma(-0.5, ke + me, U[4]);
+    V[5] = U[5]; V[6] = U[6]; V[7] = U[7]; V[8] = U[8];
+    return d_pos(V[0]) && d_pos(V[4]) ? 0u : state_flags(V[0], V[4]);
 }
 
 template <>
@@ -472,12 +481,10 @@ __device__ __forceinline__ unsigned int prim_any(const double (&U)[NV], const St
 #pragma unroll
         for (int q = 0; q < NV; ++q) V[q] = o.V[q];
         return o.st;
+    } else if constexpr (sizeof(R) == 8) {
+        return sr_prim_fp64(U, a.gam, a.sr_g1, df{a.sr_g1h, a.sr_g1l}, 0.0f, V);
     } else {
-        double Vd[NV];
-        const unsigned int st = sr_prim<R>(U, a.gam, Vd);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) V[q] = (R)Vd[q];
-        return st;
+        return 0u;  // ideal MHD in float32, above
     }
 }
 
@@ -500,9 +507,10 @@ __device__ __forceinline__ R cell_speed(const R (&V)[NV], const StepArgs &a, con
             const R bt2 = b2 - bn2;
             const R disc = sqrt((a2 - b2) * (a2 - b2) + R(4) * a2 * bt2);
             s = fabs(V[1 + d]) + sqrt(R(0.5) * (a2 + b2 + disc));
-        } else if (PHYS == PH_MHD) {
+        } else if constexpr (PHYS == PH_MHD) {
             const int b1 = 5 + (d == 0 ? 1 : 0), b2 = 5 + (d == 2 ? 1 : 2);
-            s = fabs(V[1 + d]) + fast_speed(V[0], V[4], V[5 + d], V[b1], V[b2], g);
+            s = fabs(V[1 + d]) + d_sqrt64(d_fast2(d_rcp64(V[0]), V[4], V[5 + d] * V[5 + d],
+                                                  V[b1] * V[b1] + V[b2] * V[b2], g));
         } else {
             R Vl[NV], lm, lp;
 #pragma unroll
@@ -542,7 +550,26 @@ template <class R, int IFACE64>
 __device__ __forceinline__ unsigned int interface_state(const R (&W)[NV], const R (&T)[NV], const StepArgs &a,
                                                         R (&out)[NV])
 {
-    if (IFACE64) {
+    if constexpr (sizeof(R) == 8) {
+        // the increment form: as cheap as forming and recovering E, and the
+        // pressure keeps the last bits that E would round away
+        const double rs = W[0], rho = rs + T[0], irho = d_rcp64(rho);
+        const double v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
+        const double vdm = W[1] * T[1] + W[2] * T[2] + W[3] * T[3];
+        const double dm2 = T[1] * T[1] + T[2] * T[2] + T[3] * T[3];
+        const double dke = fma(rs, fma(v2, T[0], -2.0 * vdm), -dm2) * (0.5 * irho);
+        const double dme = T[5] * fma(0.5, T[5], W[5]) + T[6] * fma(0.5, T[6], W[6]) + T[7] * fma(0.5, T[7], W[7]);
+        out[0] = rho;
+        out[1] = fma(rs, W[1], T[1]) * irho;
+        out[2] = fma(rs, W[2], T[2]) * irho;
+        out[3] = fma(rs, W[3], T[3]) * irho;
+        out[4] = fma(a.gam - 1.0, (T[4] + dke) - dme, W[4]);
+        out[5] = W[5] + T[5];
+        out[6] = W[6] + T[6];
+        out[7] = W[7] + T[7];
+        out[8] = W[8] + T[8];
+        return d_pos(rho) && d_pos(out[4]) ? 0u : state_flags(rho, out[4]);
+    } else if (IFACE64) {
         const double rho = W[0], vx = W[1], vy = W[2], vz = W[3], p = W[4];
         const double bx = W[5], by = W[6], bz = W[7];
         double U[NV], V[NV];
@@ -590,6 +617,17 @@ __device__ __forceinline__ unsigned int interface_state(const R (&W)[NV], const 
 // in them, hence the last bit of every flux.
 __host__ __device__ constexpr bool sr_df_sweep(int D) { return D == 0; }
 
+// Newton's start in float32: W = w gamma^2 of a nearby float64 state (0, no
+// guess, where 1 - v^2 is beyond float32's resolution).
+__device__ __forceinline__ float sr_w0_f(const double (&V)[NV], const StepArgs &a)
+{
+    const float vx = d2f_int(V[1]), vy = d2f_int(V[2]), vz = d2f_int(V[3]);
+    const float ev = 1.0f - (vx * vx + vy * vy + vz * vz);
+    const float rho = d2f_int(V[0]), p = d2f_int(V[4]);
+    const float w = a.gam > 0.0 ? rho + a.sr_igh * p : 2.5f * p + sqrtf(2.25f * p * p + rho * rho);
+    return ev > 1.0e-6f ? w / ev : 0.0f;
+}
+
 // SRMHD interface state at n+1/2: U(V*) + T formed in float64, recovered by
 // the float64 Newton iteration (Eq. transv).
 template <class R, int D>
@@ -607,12 +645,18 @@ __device__ __forceinline__ unsigned int sr_interface(const R (&W)[NV], const R (
 #pragma unroll
         for (int q = 0; q < NV; ++q) out[q] = o.V[q];
         return o.st;
-    } else {
+    } else if constexpr (sizeof(R) == 4) {
         double V[NV];
         const unsigned int st = sr_interface64<R>(W, T, a.gam, V);
 #pragma unroll
         for (int q = 0; q < NV; ++q) out[q] = (R)V[q];
         return st;
+    } else {
+        double U[NV];
+        sr_cons<double, double>(W, a.gam, U);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) U[q] += T[q];
+        return sr_prim_fp64(U, a.gam, a.sr_g1, df{a.sr_g1h, a.sr_g1l}, sr_w0_f(W, a), out);
     }
 }
 
@@ -659,7 +703,20 @@ __device__ __forceinline__ unsigned int trace_cell_t(const StepArgs &a, const De
             double U0[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q) U0[q] = a.U[gperm<D>(q) * a.ustride + gi];
-            f |= sr_mh_predict<R>(vs[1], vs[2], vs[3], U0, pgam<R>(a), ch, dtdx, a.gam, pl, ml);
+            if constexpr (sizeof(R) == 4) {
+                f |= sr_mh_predict<R>(vs[1], vs[2], vs[3], U0, pgam<R>(a), ch, dtdx, a.gam, pl, ml);
+            } else {
+                R dV[NV], x[NV], Us[NV], Vh[NV];
+                sr_mh_increment<R>(vs[1], vs[2], vs[3], pgam<R>(a), ch, dtdx, dV, x);
+#pragma unroll
+                for (int q = 0; q < NV; ++q) Us[q] = U0[q] - x[q];
+                f |= sr_prim_fp64(Us, a.gam, a.sr_g1, df{a.sr_g1h, a.sr_g1l}, sr_w0_f(vs[2], a), Vh);
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    pl[q] = fma(0.5, dV[q], Vh[q]);
+                    ml[q] = fma(-0.5, dV[q], Vh[q]);
+                }
+            }
         }
     }
 #pragma unroll
@@ -1156,7 +1213,7 @@ __global__ void __launch_bounds__(BLOCK) k_div1(StepArgs a, GroupTable gt, const
     const Where wh = locate(gt);
     const DevPatch P = a.patches[wh.patch];
     const Tile t(D == 0 ? wh.dx : wh.rw);
-    const int SEGL = wh.seg;
+    const int SEGL = wh.seg1;
     const R gam = pgam<R>(a), ch = pch<R>(a.sp);
     const R iD = pidx<R>(P, D);
     R *Ld = L1 + (long long)D * NV * a.sstride;
@@ -1325,7 +1382,7 @@ __global__ void __launch_bounds__(BLOCK) k_pred(StepArgs a, GroupTable gt, const
         }
     } else {
         constexpr int O = D == 1 ? 2 : 1;  // the other transverse dimension
-        const int SEGL = wh.seg;
+        const int SEGL = wh.seg1;
         const int nD = P.n[D];
         const int eO = a.ndim > O ? P.n[O] + 2 : 1, loO = a.ndim > O ? -1 : 0;
         const int nseg = (nD + SEGL - 1) / SEGL;

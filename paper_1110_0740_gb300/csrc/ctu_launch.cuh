@@ -40,6 +40,7 @@ static int over_groups(const LaunchInfo &li, BPP bpp, GO go, XR xr = XR())
             gt.bs2[k] = dm.s2;
             gt.xw[k] = G.xw;
             gt.seg[k] = G.seg;
+            gt.seg1[k] = G.seg1;
             gt.xr[k] = (unsigned char)xr(G);
             gt.sx[k] = G.sx;
             gt.dx[k] = G.dx;
@@ -173,11 +174,11 @@ static int launch_step_t(const StepArgs &a, const LaunchInfo &li, cudaStream_t s
                 li, [&](const Group &G) { return Tiles::pred_x(G.n, a.ndim, G.xw); },
                 [&](const GroupTable &gt, unsigned nb) { k_pred<PHYS, R, PPM, 0><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg1); },
                 [&](const GroupTable &gt, unsigned nb) { k_pred<PHYS, R, PPM, 1><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
             if (a.ndim > 2)
                 n += over_groups(
-                    li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg); },
+                    li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg1); },
                     [&](const GroupTable &gt, unsigned nb) {
                         k_pred<PHYS, R, PPM, 2><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1);
                     });
@@ -186,19 +187,19 @@ static int launch_step_t(const StepArgs &a, const LaunchInfo &li, cudaStream_t s
     } else if (a.ndim > 1 || EXT) {
         CTU_MARK("flux1");
         const int xr1 = launch_rows(li, DIV1X_ROWS, [&](const Group &G, int x) {
-            return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg, EXT, x);
+            return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg1, EXT, x);
         });
         n += over_groups(
-            li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg, EXT, xr1); },
+            li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 0, G.dx, G.seg1, EXT, xr1); },
             [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 0, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); },
             [&](const Group &G) { return Tiles::div1x_rows(G.n, a.ndim, G.dx, xr1); });
         if (a.ndim > 1)
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg, EXT); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 1, G.rw, G.seg1, EXT); },
                 [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 1, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
         if (a.ndim > 2)
             n += over_groups(
-                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg, EXT); },
+                li, [&](const Group &G) { return Tiles::div1(G.n, a.ndim, 2, G.rw, G.seg1, EXT); },
                 [&](const GroupTable &gt, unsigned nb) { k_div1<PHYS, R, 2, HY, HC, EXT><<<nb, BLOCK, 0, s>>>(a, gt, Vs, L1); });
         CTU_MARK(nullptr);
     }

@@ -19,13 +19,13 @@ struct ProfHook {
 };
 
 // Patches of identical shape, contiguous in the device patch table, with the
-// thread-tile width along x (8, 16 or 32), the marching segment length and the
-// row widths of the x-tiled and ring kernels (group_widths).  A launch covers
+// thread-tile width along x (8, 16 or 32), the marching segment lengths (the
+// sweeps', the first-order kernels') and the row widths of the x-tiled and ring kernels (group_widths).  A launch covers
 // up to MAXG groups (GroupTable).
 struct Group {
     int first, count;
     int n[3], N[3];
-    int xw, seg;
+    int xw, seg, seg1;
     unsigned char sx, dx, rw;
 };
 inline void group_widths(Group &G, int ndim, bool f64, bool mt)
@@ -35,24 +35,23 @@ inline void group_widths(Group &G, int ndim, bool f64, bool mt)
     G.rw = (unsigned char)ring_width(G.n, f64 ? 0.0 : mt ? 0.004 : 0.01);
 }
 
-// Marching segment length of the groups `pick` marks (the untuned ones) for a
-// batch: the candidate with the least modelled time of the launches along y
-// and z.  A thread marches L = seg + 2 cells (two are its neighbours'), so
-// long segments do the least work, but a small batch then leaves most of the
-// chip idle behind a few serial chains.  With B blocks on S SMs, a step of
-// the march takes a + k while k blocks share an SM (a: the latency part, in
-// units of the throughput part of one block), 3 blocks of the sweeps' 168
-// registers fit, and the whole launch L times
-//   floor(B / 3S) (a + 3) + (a + ceil(rest / S), if a rest is left).
+// Marching segment lengths for a batch: of the first-order kernels (seg1) and,
+// for the groups `pick` marks (the untuned ones), of the sweeps (seg), each the
+// candidate with the least modelled time of its launches along y and z.  A
+// thread marches L = seg + 2 cells (seg + 1), so long segments do the least
+// work, but a small batch then leaves most of the chip idle behind a few
+// serial chains.  With B blocks on S SMs, a step of the march takes a + k
+// while k blocks share an SM (a: the latency part, in units of the throughput
+// part of one block), at most `fit` of them, and the whole launch L times
+//   floor(B / (fit S)) (a + fit) + (a + ceil(rest / S), if a rest is left).
 // Fitted on the GB300 to 11 lengths of 21 shapes: a = 1.5 in float32 and for
 // relativistic flow, 0.15 for float64 MHD, whose single block per SM already
-// fills the FP64 pipe; the model picks the fastest or one within 4%.  The
-// first-order kernels march L - 1 cells at 0.3 of a sweep's cost, five blocks
-// to an SM in float32.  Relativistic pencils differ much in their iterations,
-// so a long one finishes late: 6 L more (128^3 beam: 19.7 ms at 6 cells, 20.0 at 8,
-// 22.8 at 16; 256^3: 16 beats 8 by 8%).  us per step at the fixed 16 and at the model's choice:
-// 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and 112, 64^3 mixed 208 and
-// 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
+// fills the FP64 pipe; the model picks the fastest or one within 4%.
+// Relativistic pencils differ much in their iterations, so a long one
+// finishes late: 6 L more (128^3 beam: 19.7 ms at 6 cells, 20.0 at 8, 22.8 at 16;
+// 256^3: 16 beats 8 by 8%).  us per step at the fixed 16 and at the model's
+// choice: 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and 112, 64^3 mixed 208
+// and 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
 template <class Pick>
 inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int sms, Pick pick)
 {
@@ -60,38 +59,37 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int 
     const double a = f64 && !rel ? 0.15 : 1.5;
     const double S = sms > 0 ? sms : 152;
     if (ndim < 2) return;
-    auto launch = [&](double blocks, double steps, double fit) {
-        if (blocks <= 0.0) return 0.0;
-        const double k = blocks / S, full = (double)(long long)(k / fit), rest = k - full * fit;
-        const double tail = rest > 0.0 ? a + (double)(long long)(rest + 0.999999) : 0.0;
-        return steps / blocks * (full * (a + fit) + tail);
-    };
-    int best = 0;
-    double top = 0.0;
-    for (int c : cand) {
-        double t = 0.0;
-        for (int D = 1; D < ndim; ++D) {
-            double b1 = 0.0, s1 = 0.0, b2 = 0.0, s2 = 0.0;
-            for (int i = 0; i < ng; ++i) {
-                const Group &G = g[i];
-                const int seg = pick(G) ? c : G.seg, len = seg < G.n[D] ? seg : G.n[D];
-                const double m = (double)G.count * Tiles::sweep_m(G.n, D, G.xw, seg);
-                const double f = (double)G.count * Tiles::div1(G.n, ndim, D, G.rw, seg);
-                b1 += m;
-                s1 += m * (len + 2);
-                b2 += f;
-                s2 += f * (len + 1);
+    for (int ring = 0; ring < 2; ++ring) {
+        // the kernels' registers: 168 (three blocks), the float first-order
+        // ones about 95 (five)
+        const double fit = ring && !f64 ? 5.0 : 3.0;
+        int best = 0;
+        double top = 0.0;
+        for (int c : cand) {
+            double t = 0.0;
+            for (int D = 1; D < ndim; ++D) {
+                double blocks = 0.0, steps = 0.0;
+                for (int i = 0; i < ng; ++i) {
+                    const Group &G = g[i];
+                    const int seg = ring || pick(G) ? c : G.seg, len = seg < G.n[D] ? seg : G.n[D];
+                    const double b = (double)G.count * (ring ? Tiles::div1(G.n, ndim, D, G.rw, seg)
+                                                             : Tiles::sweep_m(G.n, D, G.xw, seg));
+                    blocks += b;
+                    steps += b * (len + (ring ? 1 : 2));
+                }
+                if (blocks <= 0.0) continue;
+                const double k = blocks / S, full = (double)(long long)(k / fit), rest = k - full * fit;
+                const double tail = rest > 1e-9 ? a + (double)(long long)(rest + 0.999999) : 0.0;
+                t += steps / blocks * (full * (a + fit) + tail + (rel && !ring ? 6.0 : 0.0));
             }
-            if (rel) t += 6.0 * s1 / b1;
-            t += launch(b1, s1, 3.0) + 0.3 * launch(b2, s2, f64 ? 3.0 : 5.0);
+            if (best == 0 || t < top) {
+                top = t;
+                best = c;
+            }
         }
-        if (best == 0 || t < top) {
-            top = t;
-            best = c;
-        }
+        for (int i = 0; i < ng; ++i)
+            if (ring || pick(g[i])) (ring ? g[i].seg1 : g[i].seg) = best;
     }
-    for (int i = 0; i < ng; ++i)
-        if (pick(g[i])) g[i].seg = best;
 }
 
 struct LaunchInfo {

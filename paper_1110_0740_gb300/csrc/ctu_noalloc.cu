@@ -129,7 +129,7 @@ extern "C" ctu_status ctu_step_noalloc(const ctu_config *cfg, const double *U_in
             groups[i].N[d] = q.N[d];
         }
         groups[i].xw = Tiles::xw(q.n[0]);
-        groups[i].seg = SEG;
+        groups[i].seg = groups[i].seg1 = SEG;
         group_widths(groups[i], cfg->ndim, cfg->precision == CTU_FP64, false);
     }
     const size_t elt = cfg->precision == CTU_FP64 ? sizeof(double) : sizeof(float);

@@ -217,11 +217,20 @@ __device__ __forceinline__ void trace(R wp, R w0, R wm, R nu, int mode, R numax,
 // positive factor, with the inverse factor on its right eigenvector;
 // reconstruction and tracing are positively homogeneous, so the result is
 // unchanged.
+// In float64, for the kinds without reference states: char_predict64
+// (mhd_fp64.cuh), the same predictor for the FP64 pipe.
+template <int PPM>
+__device__ __forceinline__ void char_predict64(const double (&vs)[5][NV], double gam, double ch, double dtdx, int upwind,
+                                               int lim, double (&Vp)[NV], double (&Vm)[NV]);
 template <class R, int PPM>
 __device__ __forceinline__ void char_predict(const R (&vs)[5][NV], R gam, R ch, R dtdx, int upwind, int lim,
                                              R dx2, R (&Vp)[NV], R (&Vm)[NV])
 {
     constexpr bool REF = PPM >= RECON_LIN && PPM <= RECON_MC_REF;
+    if constexpr (sizeof(R) == 8 && !REF) {
+        char_predict64<PPM>(vs, gam, ch, dtdx, upwind, lim, Vp, Vm);
+        return;
+    }
     const R rho = vs[2][0], u = vs[2][1], v1c = vs[2][2], v2c = vs[2][3], pc = vs[2][4];
     const R Bn = vs[2][5], B1c = vs[2][6], B2c = vs[2][7];
     const R a2 = gam * pc / rho;

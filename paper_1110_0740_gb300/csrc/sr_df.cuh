@@ -30,6 +30,7 @@
 // error-free transformations.
 #pragma once
 
+#include "mhd_fp64.cuh"
 #include "srmhd_device.cuh"
 
 namespace ctu {
@@ -464,6 +465,148 @@ __device__ __forceinline__ unsigned int sr_mh_predict_f(const float (&vm1)[NV], 
         Vm[q] = V[q] - 0.5f * dV[q];
     }
     return st;
+}
+
+// ---- the FP64 path
+
+// W of the energy equation to double-float accuracy (about 1e-13 relative): the
+// float32 Newton steps, bracketed where they leave the physical range, then
+// double-float steps until one moves W by less than 1e-7.  No certificate: a
+// start for the float64 step.  false: not found.
+__device__ __forceinline__ bool sr_seed(const SrState &u, float W0, df g1, double &Wd)
+{
+    const df m2 = d_addp(d_addp(d_sqr(u.m[0]), d_sqr(u.m[1])), d_sqr(u.m[2]));
+    const df B2 = d_addp(d_addp(d_sqr(u.b[0]), d_sqr(u.b[1])), d_sqr(u.b[2]));
+    const df S = d_add(d_add(d_mul(u.m[0], u.b[0]), d_mul(u.m[1], u.b[1])), d_mul(u.m[2], u.b[2]));
+    if (!(u.D.hi > 0.0f) || !(u.tau.hi > 0.0f)) return false;
+    if (!(W0 > 0.0f)) W0 = d_add(u.tau, d_neg(d_half(B2))).hi;
+    const float S2f = d_sqr(S).hi;
+    float Wf = W0;
+    bool in = W0 > 0.0f;
+    for (int it = 0; it < 8 && in; ++it) {
+        float f, dfw;
+        in = sr_energy_f(Wf, u.D.hi, m2.hi, S2f, B2.hi, u.tau.hi, g1.hi, f, dfw);
+        const float Wn = Wf - f / dfw;
+        in = in && Wn > 0.0f;
+        const bool done = fabsf(Wn - Wf) <= 1.0e-5f * Wf;
+        if (in) Wf = Wn;
+        if (done) break;
+    }
+    if (!in) Wf = sr_bracket_f(u.D.hi, m2.hi, S2f, B2.hi, u.tau.hi, g1.hi);
+    df W{Wf, 0.0f};
+    const df hB = d_half(B2);
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+        const df Wb = d_addp(W, B2), iW = d_rcp(W), iWb = d_rcp(Wb);
+        const df t2 = d_sqr(d_mul(S, iW));
+        const df v2 = d_mul(d_addp(m2, d_mul(t2, d_addp(W, Wb))), d_sqr(iWb));
+        const df ev = d_addf(d_neg(v2), 1.0f);
+        if (!(ev.hi > 0.0f)) return false;
+        const df is = d_rsqrt(ev);
+        const df p = d_mul(g1, d_add(d_mul(W, ev), d_neg(d_mul(u.D, d_mul(ev, is)))));
+        const df f = d_add(d_add(d_add(d_add(W, d_neg(u.tau)), hB), d_mul(hB, v2)), d_neg(d_add(p, d_half(t2))));
+        // f' in float32: the step's error is its square and 1e-6 of it
+        const float dv2 = -2.0f * iWb.hi * (v2.hi + t2.hi * iW.hi);
+        const float dp = g1.hi * (ev.hi + dv2 * (0.5f * u.D.hi * is.hi - W.hi));
+        const float dF = 1.0f - dp + hB.hi * dv2 + t2.hi * iW.hi;
+        const float dW = -__fdividef(f.hi, dF);
+        W = d_addf(W, dW);
+        if (!(W.hi > 0.0f)) return false;
+        if (fabsf(dW) <= 1.0e-7f * W.hi) {
+            Wd = f2d_int(W.hi) + f2d_int(W.lo);
+            return true;
+        }
+    }
+    return false;
+}
+
+struct SrOut64 {
+    double V[5];
+    unsigned int st;
+};
+
+// rho, v and p of a conserved state in float64 (ideal gas, g1 = (Gamma - 1) /
+// Gamma; the Taub-Mathews gas, gam = 0, keeps sr_prim64): W from sr_seed on the
+// FP32 pipe, so that one float64 evaluation of the energy equation remains,
+// with v^2 and p carried over its step by their first-order terms (a step of at
+// most 1e-9 W: a remainder of 1e-18).  sr_prim64 took several evaluations from
+// a guess, and its bracketed iteration tens of them for the lanes without a
+// usable one, the whole warp waiting.  64^3 beam, ms per launch before and
+// after (with the FP64 forms of the fluxes): prim 1.29 and 0.095, sweep z 7.5 and
+// 1.32, y 8.6 and 1.36, x 3.8 and 0.86.
+static __device__ __noinline__ SrOut64 sr_prim_fp64(SrCons c, double gam, double g1, df g1f, float W0)
+{
+    SrOut64 o;
+    const double D = c.U[0], tau = c.U[4] + c.U[0];
+    double W = 0.0;
+    bool ok = false;
+    if (gam > 0.0) {
+        SrState u;
+        u.D = sr_split(c.U[0]);
+        u.tau = d_add(sr_split(c.U[4]), u.D);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            u.m[k] = sr_split(c.U[1 + k]);
+            u.b[k] = sr_split(c.U[5 + k]);
+        }
+        ok = sr_seed(u, W0, g1f, W);
+    }
+    if (ok) {
+        const double m2 = c.U[1] * c.U[1] + c.U[2] * c.U[2] + c.U[3] * c.U[3];
+        const double B2 = c.U[5] * c.U[5] + c.U[6] * c.U[6] + c.U[7] * c.U[7];
+        const double S = c.U[1] * c.U[5] + c.U[2] * c.U[6] + c.U[3] * c.U[7];
+        ok = false;
+#pragma unroll 1
+        for (int it = 0; it < 3; ++it) {
+            const double Wb = W + B2, iW = d_rcp64(W), iWb = d_rcp64(Wb);
+            const double t = S * iW, t2 = t * t, t2W = t2 * iW;
+            const double v2 = fma(t2, W + Wb, m2) * (iWb * iWb);
+            const double dv2 = -2.0 * iWb * (v2 + t2W);
+            const double ev = 1.0 - v2;
+            double is, s;
+            if (!d_pos(ev)) break;
+            d_roots64(ev, is, s);
+            const double p = g1 * (W * ev - D * s);
+            const double dp = g1 * fma(dv2, fma(0.5 * D, is, -W), ev);
+            const double f = ((W - tau) + 0.5 * B2) + fma(0.5, fma(B2, v2, -t2), -p);
+            const double dF = (1.0 - dp) + fma(0.5 * B2, dv2, t2W);
+            const double dW = -f * d_rcp64(dF), Wn = W + dW;
+            if (!d_pos(Wn)) break;
+            if (d_mag(dW) <= d_mag(1.0e-9 * W)) {
+                const double evn = fma(-dv2, dW, ev), pn = fma(dp, dW, p);
+                if (!d_pos(evn)) break;
+                const double iq = d_rcp64(Wn + B2), SW = S * d_rcp64(Wn);
+                o.V[0] = D * d_sqrt64(evn);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) o.V[1 + k] = fma(SW, c.U[5 + k], c.U[1 + k]) * iq;
+                o.V[4] = pn;
+                o.st = d_pos(o.V[0]) && d_pos(pn) ? 0u : 1u;
+                ok = true;
+                break;
+            }
+            W = Wn;
+        }
+    }
+    if (!ok) {
+        double V[NV];
+        o.st = sr_prim64(c.U, gam, V, f2d_int(W0));
+#pragma unroll
+        for (int q = 0; q < 5; ++q) o.V[q] = V[q];
+    }
+    return o;
+}
+__device__ __forceinline__ unsigned int sr_prim_fp64(const double (&U)[NV], double gam, double g1, df g1f, float W0,
+                                                     double (&V)[NV])
+{
+    SrCons c;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) c.U[q] = U[q];
+    const SrOut64 o = sr_prim_fp64(c, gam, g1, g1f, W0);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) V[q] = o.V[q];
+#pragma unroll
+    for (int q = 5; q < NV; ++q) V[q] = U[q];
+    return o.st;
 }
 
 } // namespace ctu

@@ -15,6 +15,7 @@
 
 #include "df.cuh"
 #include "mhd_device.cuh"
+#include "mhd_fp64.cuh"
 
 namespace ctu {
 
@@ -54,6 +55,34 @@ template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return
 template <class T> __device__ __forceinline__ T sqrt_t(T x) { return x > T(0) ? x * rsqrt_t<T>(x) : T(0); }
 template <> __device__ __forceinline__ float sqrt_t<float>(float x) { return sqrtf(x); }
 
+// The same in a function of the working precision R (double: the FP64 path's
+// forms, mhd_fp64.cuh; T = double with R = float is the mixed path's float64
+// recovery, which keeps the forms above).
+template <class T, class R> __device__ __forceinline__ T inv_t(T x)
+{
+    if constexpr (sizeof(R) == 8)
+        return d_rcp64(x);
+    else
+        return rcp_t<T>(x);
+}
+template <class T, class R> __device__ __forceinline__ T rinv_t(T x)
+{
+    if constexpr (sizeof(R) == 8) {
+        double y, s;
+        d_roots64(x, y, s);
+        return y;
+    } else {
+        return rsqrt_t<T>(x);
+    }
+}
+template <class R> __device__ __forceinline__ R root_t(R x)
+{
+    if constexpr (sizeof(R) == 8)
+        return d_sqrt64(x);
+    else
+        return sqrt_t<R>(x);
+}
+
 // Enthalpy density w(rho, p): the ideal gas of Eq. (gammaEos) for gam > 0
 // (Gamma = gam), the Taub-Mathews gas of Eq. (TMEos) for gam == 0.
 template <class T> __device__ __forceinline__ T sr_w(T rho, T p, T gam)
@@ -66,7 +95,7 @@ template <class T> __device__ __forceinline__ T sr_w(T rho, T p, T gam)
 // p (5 w - 8 p) / (3 w (w - p)) (Taub-Mathews, Mignone & McKinney 2007).
 template <class T> __device__ __forceinline__ T sr_cs2(T p, T w, T gam)
 {
-    if (gam > T(0)) return gam * p / w;
+    if (gam > T(0)) return sizeof(T) == 8 ? gam * p * inv_t<T, T>(w) : gam * p / w;
     return p * (T(5) * w - T(8) * p) / (T(3) * w * (w - p));
 }
 
@@ -77,12 +106,12 @@ __device__ __forceinline__ void sr_cons(const R (&V)[NV], T gam, T (&U)[NV])
     const T rho = V[0], vx = V[1], vy = V[2], vz = V[3], p = V[4];
     const T bx = V[5], by = V[6], bz = V[7];
     const T v2 = vx * vx + vy * vy + vz * vz;
-    const T lor2 = rcp_t<T>(T(1) - v2);
+    const T lor2 = inv_t<T, R>(T(1) - v2);
     const T W = sr_w<T>(rho, p, gam) * lor2;
     const T B2 = bx * bx + by * by + bz * bz;
     const T vB = vx * bx + vy * by + vz * bz;
     const T E2 = B2 * v2 - vB * vB;
-    U[0] = rho * rsqrt_t<T>(T(1) - v2);
+    U[0] = rho * rinv_t<T, R>(T(1) - v2);
     U[1] = (W + B2) * vx - vB * bx;
     U[2] = (W + B2) * vy - vB * by;
     U[3] = (W + B2) * vz - vB * bz;
@@ -341,13 +370,13 @@ __device__ __forceinline__ void sr_speeds(const R (&V)[NV], R gam, R &lm, R &lp)
     const R rh = sr_w<R>(V[0], V[4], gam);
     const R cs2 = sr_cs2<R>(V[4], rh, gam);
     const R b2 = B2 * (R(1) - v2) + vB * vB;
-    const R ca2 = b2 * rcp_t<R>(rh + b2);
+    const R ca2 = b2 * inv_t<R, R>(rh + b2);
     const R a2 = cs2 + ca2 - cs2 * ca2;
     const R den = R(1) - v2 * a2;
     R disc = a2 * (R(1) - v2) * (R(1) - v2 * a2 - vn * vn * (R(1) - a2));
     disc = fmax(disc, R(0));
-    const R sq = sqrt_t<R>(disc);
-    const R id = rcp_t<R>(den);
+    const R sq = root_t<R>(disc);
+    const R id = inv_t<R, R>(den);
     lm = (vn * (R(1) - a2) - sq) * id;
     lp = (vn * (R(1) - a2) + sq) * id;
 }
@@ -360,7 +389,7 @@ __device__ __forceinline__ void sr_flux(const R (&V)[NV], const R (&U)[NV], R ga
     const R vx = V[1], vy = V[2], vz = V[3], p = V[4];
     const R bx = V[5], by = V[6], bz = V[7];
     const R v2 = vx * vx + vy * vy + vz * vz;
-    const R W = sr_w<R>(V[0], p, gam) * rcp_t<R>(R(1) - v2);
+    const R W = sr_w<R>(V[0], p, gam) * inv_t<R, R>(R(1) - v2);
     const R ex = -(vy * bz - vz * by), ey = -(vz * bx - vx * bz), ez = -(vx * by - vy * bx);
     const R pt = p + R(0.5) * (bx * bx + by * by + bz * bz + ex * ex + ey * ey + ez * ez);
     F[0] = U[0] * vx;
@@ -381,7 +410,7 @@ __device__ __forceinline__ void riemann_hll_sr(const R (&L0)[NV], const R (&R0)[
     R L[NV], Rt[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) { L[q] = L0[q]; Rt[q] = R0[q]; }
-    const R Bm = R(0.5) * (L[5] + Rt[5]) - R(0.5) * (Rt[8] - L[8]) * rcp_t<R>(ch);
+    const R Bm = R(0.5) * (L[5] + Rt[5]) - R(0.5) * (Rt[8] - L[8]) * inv_t<R, R>(ch);
     const R pm = R(0.5) * (L[8] + Rt[8]) - R(0.5) * ch * (Rt[5] - L[5]);
     L[5] = Bm;
     Rt[5] = Bm;
@@ -401,7 +430,7 @@ __device__ __forceinline__ void riemann_hll_sr(const R (&L0)[NV], const R (&R0)[
 #pragma unroll
         for (int q = 0; q < NV; ++q) F[q] = FR[q];
     } else {
-        const R is = rcp_t<R>(SR - SL);
+        const R is = inv_t<R, R>(SR - SL);
 #pragma unroll
         for (int q = 0; q < NV; ++q) F[q] = (SR * FL[q] - SL * FR[q] + SL * SR * (UR[q] - UL[q])) * is;
     }
@@ -419,7 +448,10 @@ __device__ __forceinline__ void sr_mh_increment(const R (&vm1)[NV], const R (&v0
     R Vpl[NV], Vmi[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-        dV[q] = mc_slope(v0[q] - vm1[q], vp1[q] - v0[q]);
+        if constexpr (sizeof(R) == 8)
+            dV[q] = d_mc64(v0[q] - vm1[q], vp1[q] - v0[q]);
+        else
+            dV[q] = mc_slope(v0[q] - vm1[q], vp1[q] - v0[q]);
         Vpl[q] = v0[q] + R(0.5) * dV[q];
         Vmi[q] = v0[q] - R(0.5) * dV[q];
     }
