@@ -611,12 +611,6 @@ __device__ __forceinline__ unsigned int interface_state(const R (&W)[NV], const 
     }
 }
 
-// Sweeps whose recoveries run in double-float (sr_df.cuh).  The others keep the
-// float64 iteration inline: their float32 fluxes are compiled around it, and
-// another shape of that code moves the fused multiply-adds the compiler picks
-// in them, hence the last bit of every flux.
-__host__ __device__ constexpr bool sr_df_sweep(int D) { return D == 0; }
-
 // Newton's start in float32: W = w gamma^2 of a nearby float64 state (0, no
 // guess, where 1 - v^2 is beyond float32's resolution).
 __device__ __forceinline__ float sr_w0_f(const double (&V)[NV], const StepArgs &a)
@@ -634,7 +628,7 @@ template <class R, int D>
 __device__ __forceinline__ unsigned int sr_interface(const R (&W)[NV], const R (&T)[NV], const StepArgs &a,
                                                      R (&out)[NV])
 {
-    if constexpr (sizeof(R) == 4 && sr_df_sweep(D)) {
+    if constexpr (sizeof(R) == 4) {
         SrFace f;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
@@ -645,12 +639,6 @@ __device__ __forceinline__ unsigned int sr_interface(const R (&W)[NV], const R (
 #pragma unroll
         for (int q = 0; q < NV; ++q) out[q] = o.V[q];
         return o.st;
-    } else if constexpr (sizeof(R) == 4) {
-        double V[NV];
-        const unsigned int st = sr_interface64<R>(W, T, a.gam, V);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) out[q] = (R)V[q];
-        return st;
     } else {
         double U[NV];
         sr_cons<double, double>(W, a.gam, U);
@@ -696,26 +684,22 @@ __device__ __forceinline__ unsigned int trace_cell_t(const StepArgs &a, const De
                              PPM == RECON_WENO3 ? R(P.dx[D] * P.dx[D]) : R(0), pl, ml);
     } else {
         const long long gi = P.base + (c - P.soff);
-        if constexpr (sizeof(R) == 4 && sr_df_sweep(D)) {
-            f |= sr_mh_predict_f(vs[1], vs[2], vs[3], a.U + gi, a.ustride, [](int q) { return gperm<D>(q); },
+        if constexpr (sizeof(R) == 4) {
+            f |= sr_mh_predict_f<D>(vs[1], vs[2], vs[3], a.U + gi, a.ustride, [](int q) { return gperm<D>(q); },
                                  pgam<R>(a), ch, dtdx, a.gam, df{a.sr_g1h, a.sr_g1l}, df{a.sr_igh, a.sr_igl}, pl, ml);
         } else {
             double U0[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q) U0[q] = a.U[gperm<D>(q) * a.ustride + gi];
-            if constexpr (sizeof(R) == 4) {
-                f |= sr_mh_predict<R>(vs[1], vs[2], vs[3], U0, pgam<R>(a), ch, dtdx, a.gam, pl, ml);
-            } else {
-                R dV[NV], x[NV], Us[NV], Vh[NV];
-                sr_mh_increment<R>(vs[1], vs[2], vs[3], pgam<R>(a), ch, dtdx, dV, x);
+            R dV[NV], x[NV], Us[NV], Vh[NV];
+            sr_mh_increment<R>(vs[1], vs[2], vs[3], pgam<R>(a), ch, dtdx, dV, x);
 #pragma unroll
-                for (int q = 0; q < NV; ++q) Us[q] = U0[q] - x[q];
-                f |= sr_prim_fp64(Us, a.gam, a.sr_g1, df{a.sr_g1h, a.sr_g1l}, sr_w0_f(vs[2], a), Vh);
+            for (int q = 0; q < NV; ++q) Us[q] = U0[q] - x[q];
+            f |= sr_prim_fp64(Us, a.gam, a.sr_g1, df{a.sr_g1h, a.sr_g1l}, sr_w0_f(vs[2], a), Vh);
 #pragma unroll
-                for (int q = 0; q < NV; ++q) {
-                    pl[q] = fma(0.5, dV[q], Vh[q]);
-                    ml[q] = fma(-0.5, dV[q], Vh[q]);
-                }
+            for (int q = 0; q < NV; ++q) {
+                pl[q] = fma(0.5, dV[q], Vh[q]);
+                ml[q] = fma(-0.5, dV[q], Vh[q]);
             }
         }
     }
@@ -766,7 +750,12 @@ __device__ __forceinline__ void face_flux(const R (&Lg)[NV], const R (&Rg)[NV], 
         L[q] = Lg[gperm<D>(q)];
         Rr[q] = Rg[gperm<D>(q)];
     }
-    if (PHYS == PH_MHD && hll)
+    if constexpr (PHYS == PH_SR && sizeof(R) == 4 && D != 0) {
+        if (gam > R(0))
+            riemann_hll_sr_m<D>(L, Rr, gam, ch, F);
+        else
+            riemann_hll_sr(L, Rr, gam, ch, F);
+    } else if (PHYS == PH_MHD && hll)
         riemann_hll(L, Rr, gam, ch, F);
     else if (PHYS == PH_MHD && HLLC)
         riemann_hllc(L, Rr, gam, ch, F);
@@ -1697,6 +1686,9 @@ __global__ void __launch_bounds__(BLOCK, CTU_MARCH_MINB) k_sweep_m(StepArgs a, G
                 } else if constexpr (FIRST) {
 #pragma unroll
                     for (int q = 0; q < NV; ++q) A[q * a.sstride + cp] = s[q];
+                } else if constexpr (PHYS == PH_SR && sizeof(R) == 4) {  // fused, see sr_side
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) A[q * a.sstride + cp] = __fmaf_rn(Fprev[q] - F[q], iD, Ap[q * as]);
                 } else {
 #pragma unroll
                     for (int q = 0; q < NV; ++q) A[q * a.sstride + cp] = Ap[q * as] + s[q];

@@ -8,10 +8,10 @@
 // the whole path at the FP64 pipe (85% busy, the FMA pipe below 3%).  A
 // double-float operation is 6 to 20 float32 ones: about a fifth of a float64
 // operation's share of its pipe.  Measured at 256^3 (beam, mixed): k_prim
-// 7.15 -> 1.30 ms, the x sweep 56.1 -> 15.4 ms.  Only the five float32 values rho, v, p leave
-// a recovery, so double-float (~2^-46) decides their rounding for all but
-// the few lanes whose value lies within the arithmetic's error of a rounding
-// boundary.  Those lanes, and every state that is not plainly physical, take
+// 7.15 -> 1.30 ms, the sweeps along z, y, x 44.8 -> 10.4, 45.4 -> 10.1,
+// 56.1 -> 15.4 ms.  Only the five float32 values rho, v, p leave a recovery,
+// so double-float (~2^-46) decides their rounding for all but the few lanes
+// whose value lies within the arithmetic's error of a rounding boundary.  Those lanes, and every state that is not plainly physical, take
 // the float64 iteration instead (the callers' noinline slow paths), so that
 // every result is the float64 iteration's, bit for bit.
 //
@@ -365,8 +365,9 @@ static __device__ __noinline__ SrOut sr_interface_slow(SrFace f, double gam)
     return o;
 }
 
-// f.V: the cell's V^n, f.T: the increment x (sr_mh_recover)
-__device__ __forceinline__ SrOut sr_mh_slow(SrCons c, SrFace f, double gam)
+// f.V: the cell's V^n, f.T: the increment x (sr_mh_recover); inline in the x
+// sweep, whose fluxes the compiler rounds around it
+__device__ __forceinline__ SrOut sr_mh_slow_in(const SrCons &c, const SrFace &f, double gam)
 {
     double V[NV];
     SrOut o;
@@ -398,6 +399,8 @@ static __device__ __noinline__ SrOut sr_interface_call(SrFace f, df g1, df ig1, 
     return sr_interface_slow(f, gam);
 }
 
+static __device__ __noinline__ SrOut sr_mh_slow(SrCons c, SrFace f, double gam) { return sr_mh_slow_in(c, f, gam); }
+
 // A float64 value as a normalised double-float.
 __device__ __forceinline__ df sr_split(double x)
 {
@@ -405,18 +408,165 @@ __device__ __forceinline__ df sr_split(double x)
     return d_norm(s.hi, s.lo);
 }
 
+// ---- float32 predictor and fluxes of the marching sweeps, every rounding
+// written out
+//
+// riemann_hll_sr and sr_mh_increment leave the choice of the fused operation
+// in sums of two products (a b + c d, which of the two is rounded first) to
+// the compiler, whose choice depends on the code around them: with another
+// recovery in the kernel the last bits of every flux move.  These forms fix
+// the choices to the ones that the sweeps along y and z were compiled to with
+// the float64 recovery inline, so that a sweep's results do not depend on what
+// else its kernel holds (the double-float recovery left to the compiler's
+// choice moved a step's output by 1.3e-8 relative; with these it is unchanged).
+// Bits by the sum they choose in (set: the second product carries the fusion,
+// the first is rounded; or, where noted, no fusion at all):
+enum : unsigned {
+    SR_V2 = 1u,   // v^2: v_x v_x + v_y v_y
+    SR_B2 = 2u,   // B^2: B_x B_x + B_y B_y
+    SR_F7 = 4u,   // v_x B_z - B_x v_z
+    SR_F4 = 8u,   // m_x - D v_x: not fused
+};
+
+// a b + c d (or, with s = -1, a b - c d), one product fused.
+template <bool SECOND> __device__ __forceinline__ float sum2(float a, float b, float c, float d, float s = 1.0f)
+{
+    return SECOND ? __fmaf_rn(s * c, d, __fmul_rn(a, b)) : __fmaf_rn(a, b, s * __fmul_rn(c, d));
+}
+
+// Conserved state, flux along the local normal (components 0..4, 6, 7) and,
+// with SPEEDS, the signal speeds of a float32 state (sr_cons, sr_flux,
+// sr_speeds; ideal gas, gw = Gamma / (Gamma - 1)).
+template <unsigned O, bool SPEEDS>
+__device__ __forceinline__ void sr_side(const float (&V)[NV], float gam, float gw, float (&U)[NV], float (&F)[NV],
+                                        float &lm, float &lp)
+{
+    const float rho = V[0], vx = V[1], vy = V[2], vz = V[3], p = V[4], bx = V[5], by = V[6], bz = V[7];
+    const float v2 = __fmaf_rn(vz, vz, sum2<(O & SR_V2) != 0>(vx, vx, vy, vy));
+    const float ev = __fadd_rn(1.0f, -v2), lor2 = __fdividef(1.0f, ev), w = __fmaf_rn(gw, p, rho);
+    const float B2 = __fmaf_rn(bz, bz, sum2<(O & SR_B2) != 0>(bx, bx, by, by));
+    const float vB = __fmaf_rn(vz, bz, sum2<false>(vx, bx, vy, by));
+    const float E2 = sum2<false>(B2, v2, vB, vB, -1.0f);
+    const float D = __fmul_rn(rho, rsqrtf(ev)), W = __fmul_rn(w, lor2), WB = __fmaf_rn(w, lor2, B2);
+    U[0] = D;
+    U[1] = sum2<false>(WB, vx, vB, bx, -1.0f);
+    U[2] = sum2<false>(WB, vy, vB, by, -1.0f);
+    U[3] = sum2<false>(WB, vz, vB, bz, -1.0f);
+    U[4] = __fadd_rn(__fmaf_rn(0.5f, __fadd_rn(B2, E2), __fmaf_rn(w, lor2, -p)), -D);
+    U[5] = bx;
+    U[6] = by;
+    U[7] = bz;
+    U[8] = V[8];
+    const float ex = -sum2<false>(vy, bz, vz, by, -1.0f), ey = -sum2<false>(vz, bx, vx, bz, -1.0f),
+                ez = -sum2<false>(vx, by, vy, bx, -1.0f);
+    const float pt = __fmaf_rn(0.5f, __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmaf_rn(ex, ex, B2))), p);
+    const float Wx = __fmul_rn(W, vx);
+    F[0] = __fmul_rn(D, vx);
+    F[1] = __fadd_rn(__fmaf_rn(-ex, ex, sum2<false>(Wx, vx, bx, bx, -1.0f)), pt);
+    F[2] = __fmaf_rn(-ex, ey, sum2<false>(Wx, vy, bx, by, -1.0f));
+    F[3] = __fmaf_rn(-ex, ez, sum2<false>(Wx, vz, bx, bz, -1.0f));
+    F[4] = (O & SR_F4) ? __fadd_rn(U[1], -F[0]) : __fmaf_rn(-D, vx, U[1]);
+    F[6] = sum2<false>(vx, by, bx, vy, -1.0f);
+    F[7] = sum2<(O & SR_F7) != 0>(vx, bz, bx, vz, -1.0f);
+    if constexpr (SPEEDS) {
+        const float cs2 = __fmul_rn(__fmul_rn(gam, p), __fdividef(1.0f, w));
+        const float b2 = sum2<false>(B2, ev, vB, vB);
+        const float ca2 = __fmul_rn(b2, __fdividef(1.0f, __fadd_rn(w, b2)));
+        const float a2 = __fmaf_rn(-cs2, ca2, __fadd_rn(cs2, ca2));
+        const float den = __fmaf_rn(-v2, a2, 1.0f), oa = __fadd_rn(1.0f, -a2);
+        const float disc = __fmul_rn(__fmul_rn(a2, ev), __fmaf_rn(-__fmul_rn(vx, vx), oa, den));
+        const float sq = sqrtf(fmaxf(disc, 0.0f)), id = __fdividef(1.0f, den);
+        lm = __fmul_rn(__fmaf_rn(vx, oa, -sq), id);
+        lp = __fmul_rn(__fmaf_rn(vx, oa, sq), id);
+    }
+}
+
+// riemann_hll_sr of the sweep along D (1 or 2).
+template <int D>
+__device__ __forceinline__ void riemann_hll_sr_m(const float (&L0)[NV], const float (&R0)[NV], float gam, float ch,
+                                                 float (&F)[NV])
+{
+    constexpr unsigned OL = SR_V2 | SR_B2 | SR_F7 | SR_F4, OR = D == 1 ? OL : OL & ~SR_V2;
+    float L[NV], R[NV], UL[NV], UR[NV], FL[NV], FR[NV], lmL, lpL, lmR, lpR;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        L[q] = L0[q];
+        R[q] = R0[q];
+    }
+    const float ich = __fdividef(1.0f, ch), gw = __fmul_rn(gam, __fdividef(1.0f, __fadd_rn(gam, -1.0f)));
+    const float Bm = __fadd_rn(__fmul_rn(0.5f, __fadd_rn(L[5], R[5])),
+                               -__fmul_rn(__fmul_rn(0.5f, __fadd_rn(R[8], -L[8])), ich));
+    const float pm = __fadd_rn(__fmul_rn(0.5f, __fadd_rn(L[8], R[8])),
+                               -__fmul_rn(__fmul_rn(0.5f, ch), __fadd_rn(R[5], -L[5])));
+    L[5] = Bm;
+    R[5] = Bm;
+    sr_side<OL, true>(L, gam, gw, UL, FL, lmL, lpL);
+    sr_side<OR, true>(R, gam, gw, UR, FR, lmR, lpR);
+    const float SL = fminf(lmL, lmR), SR = fmaxf(lpL, lpR);
+    const float is = __fdividef(1.0f, __fadd_rn(SR, -SL)), ss = __fmul_rn(SL, SR);
+    const bool left = SL >= 0.0f, right = SR <= 0.0f;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (q == 5 || q == 8) continue;
+        const float d = sum2<false>(SR, FL[q], SL, FR[q], -1.0f);
+        const float mid = __fmul_rn(__fmaf_rn(ss, __fadd_rn(UR[q], -UL[q]), d), is);
+        F[q] = left ? FL[q] : right ? FR[q] : mid;
+    }
+    F[5] = pm;
+    F[8] = __fmul_rn(__fmul_rn(ch, ch), Bm);
+}
+
+// sr_mh_increment of the sweep along D (1 or 2).
+template <int D>
+__device__ __forceinline__ void sr_mh_increment_m(const float (&vm1)[NV], const float (&v0)[NV], const float (&vp1)[NV],
+                                                  float gam, float ch, float dtdx, float (&dV)[NV], float (&x)[NV])
+{
+    constexpr unsigned OP = SR_B2 | SR_F4, OM = D == 1 ? SR_B2 | SR_F7 : SR_F7;
+    float P[NV], M[NV], UP[NV], UM[NV], FP[NV], FM[NV], l0, l1;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        dV[q] = mc_slope(__fadd_rn(v0[q], -vm1[q]), __fadd_rn(vp1[q], -v0[q]));
+        P[q] = __fmaf_rn(0.5f, dV[q], v0[q]);
+        M[q] = __fmaf_rn(-0.5f, dV[q], v0[q]);
+    }
+    const float gw = __fmul_rn(gam, __fdividef(1.0f, __fadd_rn(gam, -1.0f))), h = __fmul_rn(0.5f, dtdx);
+    sr_side<OP, false>(P, gam, gw, UP, FP, l0, l1);
+    sr_side<OM, false>(M, gam, gw, UM, FM, l0, l1);
+    const float c2 = __fmul_rn(ch, ch);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        float d;
+        if (q == 0)
+            d = sum2<true>(UP[0], P[1], UM[0], M[1], -1.0f);
+        else if (q == 5)
+            d = __fadd_rn(P[8], -M[8]);
+        else if (q == 8)
+            d = sum2<false>(c2, P[5], c2, M[5], -1.0f);
+        else
+            d = __fadd_rn(FP[q], -FM[q]);
+        x[q] = __fmul_rn(h, d);
+    }
+}
+
 // sr_mh_predict of the mixed path (global component gp(q) of the pool at Uc[
 // gp(q) us] is local component q): U* = U_i^n - x in double-float, recovered by
 // sr_recover.  B and psi of the half-step state are U*'s, rounded; where
 // double-float leaves one undecided the float64 path takes the cell.
-template <class GP>
+template <int D, class GP>
 __device__ __forceinline__ unsigned int sr_mh_predict_f(const float (&vm1)[NV], const float (&v0)[NV],
                                                         const float (&vp1)[NV], const double *Uc, long long us, GP gp,
                                                         float gam, float ch, float dtdx, double gamd, df g1, df ig1,
                                                         float (&Vp)[NV], float (&Vm)[NV])
 {
     float dV[NV], x[NV], V[NV];
-    sr_mh_increment<float>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+    if constexpr (D == 0) {
+        sr_mh_increment<float>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+    } else {
+        if (gam > 0.0f)
+            sr_mh_increment_m<D>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+        else  // the Taub-Mathews gas
+            sr_mh_increment<float>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
+    }
     unsigned int st = 0;
     bool ok = false;
     if (g1.hi > 0.0f) {
@@ -454,7 +604,7 @@ __device__ __forceinline__ unsigned int sr_mh_predict_f(const float (&vm1)[NV], 
             f.V[q] = v0[q];
             f.T[q] = x[q];
         }
-        const SrOut o = sr_mh_slow(c, f, gamd);
+        const SrOut o = D == 0 ? sr_mh_slow_in(c, f, gamd) : sr_mh_slow(c, f, gamd);
         st = o.st;
 #pragma unroll
         for (int q = 0; q < NV; ++q) V[q] = o.V[q];

@@ -479,25 +479,6 @@ __device__ __forceinline__ unsigned int sr_mh_recover(const double (&U0)[NV], co
     return sr_prim<R>(Us, gamd, Vs, Wc);
 }
 
-// MUSCL-Hancock normal predictor of one cell: V*_(+/-) = V(U*) +/- dV/2,
-// U0 = U_i^n (local, float64).
-template <class R>
-__device__ __forceinline__ unsigned int sr_mh_predict(const R (&vm1)[NV], const R (&v0)[NV], const R (&vp1)[NV],
-                                                      const double (&U0)[NV], R gam, R ch, R dtdx, double gamd,
-                                                      R (&Vp)[NV], R (&Vm)[NV])
-{
-    R dV[NV], x[NV];
-    sr_mh_increment<R>(vm1, v0, vp1, gam, ch, dtdx, dV, x);
-    double Vs[NV];
-    const unsigned int st = sr_mh_recover<R>(U0, v0, x, gamd, Vs);
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        Vp[q] = (R)Vs[q] + R(0.5) * dV[q];
-        Vm[q] = (R)Vs[q] - R(0.5) * dV[q];
-    }
-    return st;
-}
-
 // Interface state at n+1/2 in float64: V(U(W) + T), Newton from the W of the
 // predicted state (the transverse correction T is an O(dt) change).
 template <class R>
