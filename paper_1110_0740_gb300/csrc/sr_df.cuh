@@ -8,8 +8,8 @@
 // the whole path at the FP64 pipe (85% busy, the FMA pipe below 3%).  A
 // double-float operation is 6 to 20 float32 ones: about a fifth of a float64
 // operation's share of its pipe.  Measured at 256^3 (beam, mixed): k_prim
-// 7.15 -> 1.30 ms, the sweeps along z, y, x 44.8 -> 10.4, 45.4 -> 10.1,
-// 56.1 -> 15.4 ms.  Only the five float32 values rho, v, p leave a recovery,
+// 7.15 -> 0.95 ms, the sweeps along z, y, x 44.8 -> 7.9, 45.4 -> 7.9,
+// 56.1 -> 11.0 ms.  Only the five float32 values rho, v, p leave a recovery,
 // so double-float (~2^-46) decides their rounding for all but the few lanes
 // whose value lies within the arithmetic's error of a rounding boundary.  Those lanes, and every state that is not plainly physical, take
 // the float64 iteration instead (the callers' noinline slow paths), so that
@@ -101,6 +101,64 @@ __device__ __forceinline__ df d_rsqrt(df x)
     return d_norm(y, __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f))));
 }
 
+// The same operations without the final normalisation: the low part may reach a
+// few units of the high part's last place (both signs, any cancellation: the
+// error stays below about 2^-47 of the operands' magnitudes).  The recovery's
+// bounds are in these magnitudes, so it needs no more; a value is normalised
+// where it cancels by design, where its high part stands for it and where it
+// leaves.  8 operations for a sum, 4 for a product, against 20 and 7: 38.2 ->
+// 28.8 ms a step of the 256^3 beam together with the float32 derivatives below
+// (the sweeps issue at 40% with the recovery three times in each, about 2000
+// instructions; fetching them is the largest stall).
+__device__ __forceinline__ df l_add(df x, df y)
+{
+    const df s = d_two_sum(x.hi, y.hi);
+    return df{s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo))};
+}
+__device__ __forceinline__ df l_addf(df x, float y)
+{
+    const df s = d_two_sum(x.hi, y);
+    return df{s.hi, __fadd_rn(s.lo, x.lo)};
+}
+__device__ __forceinline__ df l_from1(df x)  // 1 - x, |x| <= 1, normalised
+{
+    const df s = d_norm(1.0f, -x.hi);
+    return d_norm(s.hi, __fadd_rn(s.lo, -x.lo));
+}
+__device__ __forceinline__ df l_mul(df x, df y)
+{
+    const df p = d_two_prod(x.hi, y.hi);
+    return df{p.hi, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p.lo))};
+}
+__device__ __forceinline__ df l_mulf(df x, float y)
+{
+    const df p = d_two_prod(x.hi, y);
+    return df{p.hi, __fmaf_rn(x.lo, y, p.lo)};
+}
+__device__ __forceinline__ df l_sqr(df x)
+{
+    const df p = d_two_prod(x.hi, x.hi);
+    return df{p.hi, __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, p.lo)};
+}
+// (the seeds are stepped once first: the rounding of a residual that carries
+// their two units in the last place would be 2^-46)
+__device__ __forceinline__ df l_rcp(df y)
+{
+    const float r0 = __fdividef(1.0f, y.hi), r = __fmaf_rn(r0, __fmaf_rn(-y.hi, r0, 1.0f), r0);
+    const float e = __fmaf_rn(-y.lo, r, __fmaf_rn(-y.hi, r, 1.0f));
+    return df{r, __fmul_rn(r, __fmaf_rn(e, e, e))};
+}
+__device__ __forceinline__ df l_rsqrt(df x)
+{
+    const float y0 = rsqrtf(x.hi);
+    const float y = __fmaf_rn(__fmul_rn(0.5f, y0), __fmaf_rn(__fmul_rn(-x.hi, y0), y0, 1.0f), y0);
+    const df t = l_mul(x, d_two_prod(y, y));
+    const float e = __fadd_rn(__fadd_rn(1.0f, -t.hi), -t.lo);
+    return df{y, __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)))};
+}
+
+__device__ __forceinline__ float l_f(df x) { return __fadd_rn(x.hi, x.lo); }
+
 // Whether every value within d of x rounds to x.hi (false for a nan).
 __device__ __forceinline__ bool d_certain(df x, float d)
 {
@@ -139,9 +197,10 @@ __device__ __forceinline__ void sr_w_of(const float (&V)[9], df ig1, df &ev, df 
     const float ax = fabsf(V[1]), ay = fabsf(V[2]), az = fabsf(V[3]);
     const float big = fmaxf(ax, fmaxf(ay, az));
     const float s1 = ax == big ? ay : ax, s2 = ax == big ? az : (ay == big ? az : ay);
-    ev = d_add(d_mul(d_two_sum(1.0f, -big), d_two_sum(1.0f, big)),
-               d_neg(d_addp(d_two_prod(s1, s1), d_two_prod(s2, s2))));
-    W = d_mul(d_addf(d_mulf(ig1, V[4]), V[0]), d_rcp(ev));
+    ev = l_add(l_mul(d_norm(1.0f, -big), d_norm(1.0f, big)), d_neg(l_add(d_two_prod(s1, s1), d_two_prod(s2, s2))));
+    ev = d_norm(ev.hi, ev.lo);
+    W = l_mul(l_addf(l_mulf(ig1, V[4]), V[0]), l_rcp(ev));
+    W = d_norm(W.hi, W.lo);
 }
 
 // U(V) + T of a float32 state for sr_recover; W0: its w gamma^2.
@@ -150,31 +209,40 @@ __device__ __forceinline__ void sr_state_of(const float (&V)[9], const float (&T
     df ev, W;
     sr_w_of(V, ig1, ev, W);
     W0 = W.hi;
-    const df B2 = d_addp(d_addp(d_two_prod(V[5], V[5]), d_two_prod(V[6], V[6])), d_two_prod(V[7], V[7]));
-    const df vB = d_add(d_add(d_two_prod(V[1], V[5]), d_two_prod(V[2], V[6])), d_two_prod(V[3], V[7]));
-    const df Wb = d_addp(W, B2);
-    u.D = d_addf(d_mulf(d_rsqrt(ev), V[0]), T[0]);
+    const df B2 = l_add(l_add(d_two_prod(V[5], V[5]), d_two_prod(V[6], V[6])), d_two_prod(V[7], V[7]));
+    const df vB = l_add(l_add(d_two_prod(V[1], V[5]), d_two_prod(V[2], V[6])), d_two_prod(V[3], V[7]));
+    const df Wb = l_add(W, B2);
+    u.D = l_addf(l_mulf(l_rsqrt(ev), V[0]), T[0]);
+    u.D = d_norm(u.D.hi, u.D.lo);
     // W - p + (B^2 (1 + v^2) - (v.B)^2) / 2, with 1 + v^2 = 2 - (1 - v^2)
-    const df q = d_add(d_mul(B2, d_addf(d_neg(ev), 2.0f)), d_neg(d_sqr(vB)));
-    u.tau = d_add(d_add(d_addf(W, -V[4]), d_half(q)), d_two_sum(T[4], T[0]));
+    const df q = l_add(l_mul(B2, l_addf(d_neg(ev), 2.0f)), d_neg(l_sqr(vB)));
+    u.tau = l_add(l_add(l_addf(W, -V[4]), d_half(q)), d_two_sum(T[4], T[0]));
+    u.tau = d_norm(u.tau.hi, u.tau.lo);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        u.m[k] = d_addf(d_add(d_mulf(Wb, V[1 + k]), d_neg(d_mulf(vB, V[5 + k]))), T[1 + k]);
+        u.m[k] = l_addf(l_add(l_mulf(Wb, V[1 + k]), d_neg(l_mulf(vB, V[5 + k]))), T[1 + k]);
         u.b[k] = d_two_sum(V[5 + k], T[5 + k]);
     }
 }
 
 // Error bounds of sr_recover, in units of 2^-48: K times the sums of the
-// magnitudes that enter 1 - v^2, the energy equation and the velocities.
-// With all three K = 1 no value out of 2e7 beam, ambient, magnetised and
-// random states rounded differently from the float64 iteration's (with 0.3,
-// 2e-5 of them did); K = 3 leaves 0.4% of the beam's and 0.1% of the
-// ambient's states to the float64 path.
+// magnitudes that enter 1 - v^2, the energy equation and the velocities; and,
+// in units of 2^-24, K_D times the float32 Newton derivatives' terms and the
+// step (2e-7 W as a rule).  With K = 3 and K_D = 2 no value out of 4e7 beam,
+// beam-edge, ambient, magnetised and random states rounded differently from the
+// float64 iteration's, also with the hardware's seeds (1/x, 1/sqrt x) off by
+// two units in the last place; with K = 1 one in 2e6 edge states did.  The
+// float64 path is left 0.6% of the beam's, 1.5% of its edge's and 0.03% of the
+// ambient's states.
 constexpr float SR_MARGIN = 1.0f / 281474976710656.0f;  // 2^-48
 #ifndef SR_K
 #define SR_K 3.0f
 #endif
 constexpr float SR_K_EV = SR_K, SR_K_F = SR_K, SR_K_V = SR_K;
+#ifndef SR_KD
+#define SR_KD 2.0f
+#endif
+constexpr float SR_K_D = SR_KD * 16777216.0f;  // in units of 2^-24 of the step
 
 // W from the energy equation in float32, as sr_prim64's bracketed iteration:
 // an upper bound by doubling from tau, then Newton steps, bisection outside
@@ -216,10 +284,13 @@ struct SrRec {
 };
 __device__ __forceinline__ bool sr_recover_in(const SrState &u, float W0, df g1, float (&V)[5])
 {
-    const df m2 = d_addp(d_addp(d_sqr(u.m[0]), d_sqr(u.m[1])), d_sqr(u.m[2]));
-    const df B2 = d_addp(d_addp(d_sqr(u.b[0]), d_sqr(u.b[1])), d_sqr(u.b[2]));
-    const df sx = d_mul(u.m[0], u.b[0]), sy = d_mul(u.m[1], u.b[1]), sz = d_mul(u.m[2], u.b[2]);
-    const df S = d_add(d_add(sx, sy), sz);
+    df m2 = l_add(l_add(l_sqr(u.m[0]), l_sqr(u.m[1])), l_sqr(u.m[2]));
+    df B2 = l_add(l_add(l_sqr(u.b[0]), l_sqr(u.b[1])), l_sqr(u.b[2]));
+    const df sx = l_mul(u.m[0], u.b[0]), sy = l_mul(u.m[1], u.b[1]), sz = l_mul(u.m[2], u.b[2]);
+    df S = l_add(l_add(sx, sy), sz);
+    m2 = d_norm(m2.hi, m2.lo);
+    B2 = d_norm(B2.hi, B2.lo);
+    S = d_norm(S.hi, S.lo);
     const float Sa = fabsf(sx.hi) + fabsf(sy.hi) + fabsf(sz.hi);
     if (!(u.D.hi > 0.0f) || !(u.tau.hi > 0.0f)) return false;
     if (!(W0 > 0.0f)) W0 = d_add(u.tau, d_neg(d_half(B2))).hi;
@@ -254,47 +325,60 @@ __device__ __forceinline__ bool sr_recover_in(const SrState &u, float W0, df g1,
     df W{Wf, 0.0f};
 #pragma unroll 1
     for (int it = 0; it < 3; ++it) {
-        const df Wb = d_addp(W, B2), A = d_addp(W, Wb);
-        const df iW = d_rcp(W), iWb = d_rcp(Wb);
-        const df t = d_mul(S, iW), t2 = d_sqr(t);
-        const df iWb2 = d_sqr(iWb);
-        const df v2 = d_mul(d_addp(m2, d_mul(t2, A)), iWb2);
-        const df t2W = d_mul(t2, iW);
-        const df dv2 = d_mul(d_addp(v2, t2W), df{-2.0f * iWb.hi, -2.0f * iWb.lo});
-        const df ev = d_addf(d_neg(v2), 1.0f);
+        const df Wb = l_add(W, B2), A = l_add(W, Wb);
+        const df iW = l_rcp(W), iWb = l_rcp(Wb);
+        const df t = l_mul(S, iW), t2 = l_sqr(t);
+        const df iWb2 = l_sqr(iWb);
+        const df v2 = l_mul(l_add(m2, l_mul(t2, A)), iWb2);
+        if (!(v2.hi <= 1.0f)) return false;
+        const df ev = l_from1(v2);
         if (!(ev.hi > 0.0f)) return false;
-        const df is = d_rsqrt(ev);
-        const df Ds = d_mul(u.D, d_mul(ev, is));
-        const df p = d_mul(g1, d_add(d_mul(W, ev), d_neg(Ds)));
-        const df dp = d_mul(g1, d_add(ev, d_mul(dv2, d_add(d_half(d_mul(u.D, is)), d_neg(W)))));
+        const df is = l_rsqrt(ev), s = l_mul(ev, is);
+        const df Ds = l_mul(u.D, s);
+        const df p = l_mul(g1, l_add(l_mul(W, ev), d_neg(Ds)));
         const df hB = d_half(B2);
         // f = W - p + B^2 (1 + v^2)/2 - t^2/2 - tau
-        const df f = d_add(d_add(d_add(d_add(W, d_neg(u.tau)), hB), d_mul(hB, v2)), d_neg(d_add(p, d_half(t2))));
-        const df dF = d_addf(d_add(d_add(d_neg(dp), d_mul(hB, dv2)), t2W), 1.0f);
-        const df dW = d_neg(d_mul(f, d_rcp(dF)));
-        const df Wn = d_add(W, dW);
+        df f = l_add(l_add(l_add(l_add(W, d_neg(u.tau)), hB), l_mul(hB, v2)), d_neg(l_add(p, d_half(t2))));
+        f = d_norm(f.hi, f.lo);
+        // derivatives and the step in float32: their relative error is of the
+        // step, which is a few 2^-24 of W (e_d below)
+        const float iWf = l_f(iW), iWbf = l_f(iWb), isf = l_f(is), v2f = l_f(v2);
+        const float t2W = l_f(t2) * iWf, dv2 = -2.0f * iWbf * (v2f + t2W), Dis = u.D.hi * isf;
+        const float dp = g1.hi * (ev.hi + dv2 * (0.5f * Dis - W.hi));
+        const float dF = 1.0f - dp + hB.hi * dv2 + t2W;
+        const float rF = __fdividef(1.0f, dF), dW0 = __fmul_rn(-f.hi, rF);
+        const float dW = __fmaf_rn(rF, __fmaf_rn(-dW0, dF, -f.hi), dW0);
+        const df Wn = l_addf(W, dW);
         if (!(Wn.hi > 0.0f)) return false;
-        const float a = fabsf(dW.hi), lim = accept * W.hi;
+        const float a = fabsf(dW), lim = accept * W.hi;
         if (a > 0.9999f * lim) {
             if (!(a > 1.0001f * lim)) return false;
-            W = Wn;
+            W = d_norm(Wn.hi, Wn.lo);
             continue;
         }
-        const df evn = d_add(ev, d_neg(d_mul(dv2, dW)));
-        const df pn = d_add(p, d_mul(dp, dW));
-        if (!(evn.hi > 0.0f)) return false;
-        const df iWbn = d_rcp(d_addp(Wn, B2)), SW = d_mul(S, d_rcp(Wn));
-        const df rho = d_mul(u.D, d_mul(evn, d_rsqrt(evn)));
+        // (1 - v^2, its root, 1/W and 1/(W + B^2) follow the step by their
+        // series in it)
+        const float dev = -dv2 * dW, h = 0.5f * dev * isf * isf;
+        const float evn = ev.hi + dev;
+        if (!(evn > 0.0f) || !(fabsf(h) <= 3.0e-4f)) return false;
+        df pn = l_addf(p, dp * dW);
+        pn = d_norm(pn.hi, pn.lo);
+        const float c = dW * iWf, cb = dW * iWbf;
+        const df iWbn = df{iWb.hi, __fmaf_rn(iWb.hi, cb * cb - cb, iWb.lo)};
+        const df SW = l_mul(S, df{iW.hi, __fmaf_rn(iW.hi, c * c - c, iW.lo)});
+        df rho = l_mul(u.D, df{s.hi, __fmaf_rn(s.hi, h - 0.5f * h * h * (1.0f - h), s.lo)});
+        rho = d_norm(rho.hi, rho.lo);
         if (!(rho.hi > 0.0f) || !(pn.hi > 0.0f)) return false;
         // error bounds (absolute), see SR_MARGIN
-        const float Ta = Sa * iW.hi, v2b = (m2.hi + Ta * Ta * A.hi) * iWb2.hi;
-        const float e_ev = SR_K_EV * v2b, Dis = u.D.hi * is.hi;
+        const float Ta = Sa * iW.hi, v2b = (m2.hi + Ta * Ta * A.hi) * iWb2.hi, e_d = SR_K_D * a;
+        const float e_ev = SR_K_EV * v2b, adv = fabsf(dv2);
         const float e_p0 = g1.hi * ((W.hi + 0.5f * Dis) * e_ev + 2.0f * SR_K_F * Ds.hi);
         const float e_f = e_p0 + hB.hi * e_ev + SR_K_F * (W.hi + B2.hi + 0.5f * Ta * Ta + u.tau.hi);
-        const float e_W = e_f / fabsf(dF.hi);
-        const float e_evn = e_ev + fabsf(dv2.hi) * e_W;
+        const float ddp = g1.hi * (ev.hi + adv * (0.5f * Dis + W.hi));
+        const float e_W = (e_f + e_d * (1.0f + ddp + hB.hi * adv + t2W)) / fabsf(dF);
+        const float e_evn = e_ev + adv * (e_W + e_d);
         const bool sure =
-            d_certain(pn, SR_MARGIN * (e_p0 + fabsf(dp.hi) * e_W)) &&
+            d_certain(pn, SR_MARGIN * (e_p0 + fabsf(dp) * e_W + ddp * e_d)) &&
             d_certain(rho, SR_MARGIN * (0.5f * Dis * e_evn + SR_K_V * rho.hi));
         if (!sure) return false;
         V[0] = rho.hi;
@@ -304,10 +388,11 @@ __device__ __forceinline__ bool sr_recover_in(const SrState &u, float W0, df g1,
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const df sb = d_mul(SW, u.b[k]);
-            const df v = d_mul(d_add(u.m[k], sb), iWbn);
+            const df sb = l_mul(SW, u.b[k]);
+            df v = l_mul(l_add(u.m[k], sb), iWbn);
+            v = d_norm(v.hi, v.lo);
             const float bi = fabsf(u.b[k].hi);
-            const float e_v = SR_K_V * (fabsf(u.m[k].hi) + Ta * bi) + (fabsf(v.hi) + fabsf(SW.hi) * bi * iW.hi) * e_W;
+            const float e_v = SR_K_V * (fabsf(u.m[k].hi) + Ta * bi) + (fabsf(v.hi) + fabsf(SW.hi) * bi * iW.hi) * (e_W + e_d);
             const bool zero = u.m[k].hi == 0.0f && sb.hi == 0.0f && u.m[k].lo == 0.0f && sb.lo == 0.0f && Ta * bi == 0.0f;
             ok &= zero || d_certain(v, iWbn.hi * (SR_MARGIN * e_v + tiny * (1.0f + bi * bs)));
             V[1 + k] = v.hi;
