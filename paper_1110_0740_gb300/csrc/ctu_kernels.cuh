@@ -128,6 +128,9 @@ constexpr int BLOCK = 128;
 #ifndef CTU_MARCH_MINB
 #define CTU_MARCH_MINB 3
 #endif
+#ifndef CTU_MARCH_MINB_SR
+#define CTU_MARCH_MINB_SR 4
+#endif
 #ifndef CTU_SWEEPX_MINB
 #define CTU_SWEEPX_MINB 6
 #endif
@@ -241,6 +244,8 @@ __device__ __forceinline__ Where locate(const GroupTable &gt)
 }
 // The marching sweeps are latency bound: they are compiled for at least
 // CTU_MARCH_MINB resident blocks per SM (register cap 65536 / (BLOCK * MINB)),
+// the float relativistic ones for CTU_MARCH_MINB_SR (256^3 beam, z and y: 7.16
+// and 7.09 ms with three, 6.93 and 6.91 with four, 7.24 and 7.40 with five),
 // the float x sweep for CTU_SWEEPX_MINB (CTU_SWEEPX_MINB_PAR with the
 // parabolic terms, whose staging needs the registers of one block fewer).
 
@@ -1604,7 +1609,8 @@ template <class R, int MODE> __host__ __device__ constexpr int sweep_m_smem()
 // are staged in shared memory by cp.async (sweep_m_smem bytes per block);
 // double: they are prefetched into L1.
 template <int PHYS, class R, int PPM, int IFACE64, int D, int MODE>
-__global__ void __launch_bounds__(BLOCK, CTU_MARCH_MINB) k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
+__global__ void __launch_bounds__(BLOCK, PHYS == PH_SR && sizeof(R) == 4 ? CTU_MARCH_MINB_SR : CTU_MARCH_MINB)
+k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
 {
     constexpr int O = D == 1 ? 2 : 1;  // the other transverse dimension
     constexpr bool STAGED = sizeof(R) == 4;
@@ -1618,10 +1624,16 @@ __global__ void __launch_bounds__(BLOCK, CTU_MARCH_MINB) k_sweep_m(StepArgs a, G
     const int nseg = (nD + SEGL - 1) / SEGL;
     const int T0 = (P.n[0] + t.xw - 1) / t.xw;
     const int b = wh.b;
-    const int x = (b % T0) * t.xw + t.tx();
+    int x = (b % T0) * t.xw + t.tx();
     const int comb = (b / T0) * t.rows + t.ty();
-    const int o = comb / nseg, seg = comb % nseg;
+    int o = comb / nseg;
+    const int seg = comb % nseg;
     const bool ok = x < P.n[0] && o < nO;
+    // Relativistic float: a barrier a cell keeps the block's warps in step, so
+    // that they fetch the recoveries' code (more than the instruction cache
+    // holds at once) together: 256^3 beam, z and y 7.9 -> 7.16 and 7.09 ms.  Every
+    // thread of the block runs the same number of iterations, idle ones empty.
+    constexpr bool STEP = PHYS == PH_SR && STAGED;
     const R gam = pgam<R>(a), ch = pch<R>(a.sp);
     const R dtr = pdt<R>(a.sp);
     const double dtd = a.sp->dt;
@@ -1632,8 +1644,9 @@ __global__ void __launch_bounds__(BLOCK, CTU_MARCH_MINB) k_sweep_m(StepArgs a, G
     if (LAST) damp = patch_damp(a, P);
     unsigned int fl = 0;
     R mx = R(0);
-    if (ok) {
-        const int j0 = seg * SEGL, j1 = min(j0 + SEGL, nD);
+    if (STEP && !ok) x = o = 0;  // cells to point at; no iteration
+    if (ok || STEP) {
+        const int j0 = seg * SEGL, j1 = STEP && !ok ? j0 - 2 : min(j0 + SEGL, nD);
         const int st = dstr(P, D);
         int cc[3];
         cc[0] = x;
@@ -1732,7 +1745,11 @@ __global__ void __launch_bounds__(BLOCK, CTU_MARCH_MINB) k_sweep_m(StepArgs a, G
                 cp_async_commit();
             };
             issue(j0 - 1, c, (j0 - 1) & 1);
-            for (int j = j0 - 1; j <= j1; ++j, c += st) {
+            for (int j = j0 - 1; j <= (STEP ? j0 + SEGL : j1); ++j, c += st) {
+                if constexpr (STEP) {
+                    __syncthreads();
+                    if (j > j1) continue;
+                }
                 const int sg = j & 1;
                 // the stage written here was last read in iteration j - 1
                 if (j < j1)

@@ -20,8 +20,8 @@ struct ProfHook {
 
 // Patches of identical shape, contiguous in the device patch table, with the
 // thread-tile width along x (8, 16 or 32), the marching segment lengths (the
-// sweeps', the first-order kernels') and the row widths of the x-tiled and ring kernels (group_widths).  A launch covers
-// up to MAXG groups (GroupTable).
+// sweeps', the first-order kernels') and the row widths of the x-tiled and ring
+// kernels (group_widths).  A launch covers up to MAXG groups (GroupTable).
 struct Group {
     int first, count;
     int n[3], N[3];
@@ -44,25 +44,29 @@ inline void group_widths(Group &G, int ndim, bool f64, bool mt)
 // while k blocks share an SM (a: the latency part, in units of the throughput
 // part of one block), at most `fit` of them, and the whole launch L times
 //   floor(B / (fit S)) (a + fit) + (a + ceil(rest / S), if a rest is left).
-// Fitted on the GB300 to 11 lengths of 21 shapes: a = 1.5 in float32 and for
-// relativistic flow, 0.15 for float64 MHD, whose single block per SM already
-// fills the FP64 pipe; the model picks the fastest or one within 4%.
-// Relativistic pencils differ much in their iterations, so a long one
-// finishes late: 6 L more (128^3 beam: 19.7 ms at 6 cells, 20.0 at 8, 22.8 at 16;
-// 256^3: 16 beats 8 by 8%).  us per step at the fixed 16 and at the model's
-// choice: 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and 112, 64^3 mixed 208
-// and 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
+// Fitted on the GB300 to 11 lengths of 21 shapes: a = 1.5 in float32, 0.15 for
+// float64 MHD, whose single block per SM already fills the FP64 pipe; the
+// model picks the fastest or one within 4%.  us per step at the fixed 16 and at
+// the model's choice: 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and 112,
+// 64^3 mixed 208 and 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
+// Relativistic sweeps, fitted to 10 lengths of 16 boxes of the beam: a = 0.5
+// in float32 and 2 in float64, and c L more (c = 0.5, 0.75), since pencils
+// differ in their iterations and a long one finishes late; within 3% of the
+// fastest in float64, within 13% in float32 (6% on average).  us of the sweep along
+// z at 8 cells, at 16 and at the choice: 64^3 mixed 376, 580, 285; 128^3 mixed
+// 1103, 1036, 1036; 64^3 float64 1068, 1280, 1068.
 template <class Pick>
 inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int sms, Pick pick)
 {
     static const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-    const double a = f64 && !rel ? 0.15 : 1.5;
     const double S = sms > 0 ? sms : 152;
     if (ndim < 2) return;
     for (int ring = 0; ring < 2; ++ring) {
-        // the kernels' registers: 168 (three blocks), the float first-order
-        // ones about 95 (five)
-        const double fit = ring && !f64 ? 5.0 : 3.0;
+        // the kernels' registers: 168 (three blocks), the float relativistic
+        // ones 128 (four), the float first-order ones about 95 (five)
+        const double fit = f64 ? 3.0 : ring ? 5.0 : rel ? 4.0 : 3.0;
+        const double a = rel && !ring ? (f64 ? 2.0 : 0.5) : f64 && !rel ? 0.15 : 1.5;
+        const double late = rel && !ring ? (f64 ? 0.75 : 0.5) : 0.0;
         int best = 0;
         double top = 0.0;
         for (int c : cand) {
@@ -80,7 +84,7 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int 
                 if (blocks <= 0.0) continue;
                 const double k = blocks / S, full = (double)(long long)(k / fit), rest = k - full * fit;
                 const double tail = rest > 1e-9 ? a + (double)(long long)(rest + 0.999999) : 0.0;
-                t += steps / blocks * (full * (a + fit) + tail + (rel && !ring ? 6.0 : 0.0));
+                t += steps / blocks * (full * (a + fit) + tail + late);
             }
             if (best == 0 || t < top) {
                 top = t;

@@ -8,7 +8,7 @@
 // the whole path at the FP64 pipe (85% busy, the FMA pipe below 3%).  A
 // double-float operation is 6 to 20 float32 ones: about a fifth of a float64
 // operation's share of its pipe.  Measured at 256^3 (beam, mixed): k_prim
-// 7.15 -> 0.95 ms, the sweeps along z, y, x 44.8 -> 7.9, 45.4 -> 7.9,
+// 7.15 -> 0.95 ms, the sweeps along z, y, x 44.8 -> 6.7, 45.4 -> 6.7,
 // 56.1 -> 11.0 ms.  Only the five float32 values rho, v, p leave a recovery,
 // so double-float (~2^-46) decides their rounding for all but the few lanes
 // whose value lies within the arithmetic's error of a rounding boundary.  Those lanes, and every state that is not plainly physical, take
