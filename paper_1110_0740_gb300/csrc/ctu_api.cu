@@ -1088,6 +1088,25 @@ static void launch_tag(const OpTable &T, TagArgs a, bool tile, cudaStream_t s)
 
 extern "C" {
 
+// Planes a block of k_tag_tile marches: TAG_SZ, halved while the launch holds
+// fewer than two blocks an SM (each block also forms sigma in the two planes
+// beside its own, so more is better as long as the chip is full).  sigma =
+// B^2/rho, us at 16 planes and at the choice: 100 x 70 x 50 36.5 and 22.1, 33 x 200
+// x 40 36.5 and 22.2 (8 planes: 25.2 and 26.3).
+static int tag_planes(const ctu_patch *p, int npatch, int ndim, int sms)
+{
+    int sz = TAG_SZ;
+    for (; sz > 4; sz /= 2) {
+        long long b = 0;
+        for (int i = 0; i < npatch; ++i)
+            if (ndim >= 2 && p[i].n[0] >= 16)
+                b += (long long)((p[i].n[0] + TAG_TX - 1) / TAG_TX) * ((p[i].n[1] + TAG_TY - 1) / TAG_TY) *
+                     ((p[i].n[2] + sz - 1) / sz);
+        if (b >= 2LL * sms) break;
+    }
+    return sz;
+}
+
 ctu_status ctu_tag(ctu_ctx *ctx, const double *U, int64_t stride, const ctu_patch *patches, int npatch, int sigma,
                    double eps, double chi_r, unsigned char *tags, int64_t *d_count, double *chi, void *stream)
 {
@@ -1101,6 +1120,7 @@ ctu_status ctu_tag(ctu_ctx *ctx, const double *U, int64_t stride, const ctu_patc
     std::vector<TagPatch> tp[2];
     std::vector<long long> blocks[2];
     const int nd = ctx->cfg.ndim;
+    const int sz = tag_planes(patches, npatch, nd, ctx->sms);
     for (int i = 0; i < npatch; ++i) {
         TagPatch q;
         for (int d = 0; d < 3; ++d) q.n[d] = patches[i].n[d];
@@ -1108,7 +1128,7 @@ ctu_status ctu_tag(ctu_ctx *ctx, const double *U, int64_t stride, const ctu_patc
         q.base = patches[i].base;
         const bool tile = !chi && nd >= 2 && q.n[0] >= 16;
         const long long b = tile ? (long long)((q.n[0] + TAG_TX - 1) / TAG_TX) * ((q.n[1] + TAG_TY - 1) / TAG_TY) *
-                                       ((q.n[2] + TAG_SZ - 1) / TAG_SZ)
+                                       ((q.n[2] + sz - 1) / sz)
                                  : ((long long)q.n[0] * q.n[1] * q.n[2] + AMR_BLOCK - 1) / AMR_BLOCK;
         tp[tile].push_back(q);
         blocks[tile].push_back(b);
@@ -1133,6 +1153,7 @@ ctu_status ctu_tag(ctu_ctx *ctx, const double *U, int64_t stride, const ctu_patc
     const double f = tag_margin(sigma, eps, chi_r);
     TagArgs a;
     a.ndim = nd;
+    a.sz = sz;
     a.U = U;
     a.us = stride;
     a.eps = eps;

@@ -50,19 +50,28 @@ struct TagPatch {
 #endif
 constexpr int TAG_TX = 32, TAG_TY = CTU_TAG_TY, TAG_SZ = CTU_TAG_SZ, TAG_TILE = TAG_TX * TAG_TY;
 
-// float32 value of a float64 x rounded to nearest (ties away from zero) in
-// integer operations: the significand is cut to 23 bits and the first
-// dropped bit added back (a carry out of the significand moves into the
-// exponent, as the encoding intends).  |result - x| <= 2^-24 |x| for
-// 2^-126 <= |x| < 2^128 - 2^103; +-0 below 2^-126 (an absolute error under
-// 2^-126); +-Inf or NaN beyond (the callers' range checks then fail).
+// |x| in float32, x a float64 rounded to nearest (ties away from zero) in
+// integer operations (the conversion instruction runs on the FP64 pipe): the
+// exponent is clamped to float32's range, the rounding bit added to the 64-bit
+// word (a carry out of the significand moves into the exponent, as the
+// encoding intends) and the significand's bits taken across both halves.  Within
+// 2^-24 |x| for 2^-126 <= |x| < 2^128 - 2^103; a denormal pattern below 2^-126 (an
+// absolute error under 2^-126); Inf or NaN at 2^128 and beyond (the callers'
+// range checks then fail).  ABS = false: for x that has to be positive, a
+// negative one becomes a denormal.
+template <bool ABS> __device__ __forceinline__ float f32_mag(double x)
+{
+    int hi = __double2hiint(x);
+    if (ABS) hi &= 0x7FFFFFFF;
+    hi = min(max(hi, 896 << 20), 1151 << 20);
+    const unsigned long long w =
+        (((unsigned long long)(unsigned)hi << 32) | (unsigned)__double2loint(x)) + 0x10000000ull;
+    return __uint_as_float(__funnelshift_l((unsigned)w, (unsigned)(w >> 32), 3) - (384u << 23));
+}
+// The same with x's sign.
 __device__ __forceinline__ float f32_rn(double x)
 {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned a = hi & 0x7FFFFFFFu, sg = hi & 0x80000000u;
-    const unsigned mag = (((a - (896u << 20)) << 3) | (lo >> 29)) + ((lo >> 28) & 1u);
-    const unsigned r = a >= (1151u << 20) ? 0x7FC00000u : (a < (897u << 20) ? sg : (sg | mag));
-    return __uint_as_float(r);
+    return __uint_as_float(__float_as_uint(f32_mag<true>(x)) | ((unsigned)__double2hiint(x) & 0x80000000u));
 }
 
 template <int KIND>
@@ -77,24 +86,57 @@ __device__ __forceinline__ double tag_sigma64(const double *U, long long us, lon
     return __ddiv_rn(U[4 * us + c], U[c]);
 }
 
-// sigma in float32 from truncated inputs; NaN where an intermediate would
-// lose its relative accuracy (denormal or overflow).
+// n / d, d normal, n zero or in [1e-30, 1e30] by magnitude: the hardware
+// reciprocal's quotient and its residual once, within 2^-24 (1 + 2^-20) of
+// the exact one.
+__device__ __forceinline__ float tag_quot(float n, float d)
+{
+    const float r = __fdividef(1.0f, d), q = __fmul_rn(n, r);
+    return __fmaf_rn(__fmaf_rn(-q, d, n), r, q);
+}
+
+// The float64 inputs of a cell's sigma, and sigma in float32 from them; NaN
+// where an intermediate would lose its relative accuracy (denormal or
+// overflow).
+template <int KIND> struct TagRaw {
+    double v[KIND == 2 ? 4 : KIND == 3 ? 2 : 1];
+};
+template <int KIND>
+__device__ __forceinline__ void tag_load(const double *U, long long us, long long c, TagRaw<KIND> &w)
+{
+    if (KIND == 1) {
+        w.v[0] = U[4 * us + c];
+    } else {
+        w.v[0] = U[c];
+        if (KIND == 2) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) w.v[(KIND == 2 ? 1 : 0) * (1 + k)] = U[(5 + k) * us + c];
+        }
+        if (KIND == 3) w.v[KIND == 3 ? 1 : 0] = U[4 * us + c];
+    }
+}
+template <int KIND> __device__ __forceinline__ float tag_conv(const TagRaw<KIND> &w)
+{
+    if (KIND <= 1) return f32_rn(w.v[0]);
+    const float r = f32_mag<false>(w.v[0]);
+    const bool rok = r >= 1e-30f && r <= 1e30f;
+    if (KIND == 2) {
+        const float b0 = f32_mag<true>(w.v[KIND == 2 ? 1 : 0]), b1 = f32_mag<true>(w.v[KIND == 2 ? 2 : 0]),
+                    b2 = f32_mag<true>(w.v[KIND == 2 ? 3 : 0]);
+        const float bb = __fadd_rn(__fadd_rn(__fmul_rn(b0, b0), __fmul_rn(b1, b1)), __fmul_rn(b2, b2));
+        const bool ok = rok && (bb == 0.0f || (bb >= 1e-30f && bb <= 1e30f));
+        return ok ? tag_quot(bb, r) : __uint_as_float(0x7FC00000u);
+    }
+    const float e = f32_rn(w.v[KIND == 3 ? 1 : 0]);
+    const bool ok = rok && (e == 0.0f || (fabsf(e) >= 1e-30f && fabsf(e) <= 1e30f));
+    return ok ? tag_quot(e, r) : __uint_as_float(0x7FC00000u);
+}
 template <int KIND>
 __device__ __forceinline__ float tag_sigma32(const double *U, long long us, long long c)
 {
-    if (KIND == 0) return f32_rn(U[c]);
-    if (KIND == 1) return f32_rn(U[4 * us + c]);
-    const float r = f32_rn(U[c]);
-    const bool rok = r >= 1e-30f && r <= 1e30f;
-    if (KIND == 2) {
-        const float b0 = f32_rn(U[5 * us + c]), b1 = f32_rn(U[6 * us + c]), b2 = f32_rn(U[7 * us + c]);
-        const float bb = __fadd_rn(__fadd_rn(__fmul_rn(b0, b0), __fmul_rn(b1, b1)), __fmul_rn(b2, b2));
-        const bool ok = rok && (bb == 0.0f || (bb >= 1e-30f && bb <= 1e30f));
-        return ok ? __fdiv_rn(bb, r) : __uint_as_float(0x7FC00000u);
-    }
-    const float e = f32_rn(U[4 * us + c]);
-    const bool ok = rok && (e == 0.0f || (fabsf(e) >= 1e-30f && fabsf(e) <= 1e30f));
-    return ok ? __fdiv_rn(e, r) : __uint_as_float(0x7FC00000u);
+    TagRaw<KIND> w;
+    tag_load<KIND>(U, us, c, w);
+    return tag_conv<KIND>(w);
 }
 
 // One direction's float32 terms; R out of range (or NaN) clears ok.
@@ -133,6 +175,7 @@ struct TagArgs {
     const TagPatch *tp;
     BlockMap map;
     int ndim;
+    int sz;  // planes of a k_tag_tile block, at most TAG_SZ
     const double *U;
     long long us;
     double eps, chi_r;
@@ -218,16 +261,20 @@ __global__ void __launch_bounds__(AMR_BLOCK) k_tag_flat(TagArgs a)
     tag_flush(a, P.slot, acc);
 }
 
-// A 32 x 8 tile of one plane per block, marching TAG_SZ planes along z.
+// A 32 x 8 tile of one plane per block, marching a.sz planes along z.
 // Two shared-memory buffers hold sigma of consecutive planes with a
 // one-cell halo in x and y; each thread carries sigma of its column at
-// z - 1, z, z + 1 and z + 2, and the halo threads the next plane's halo
-// value, so the loads of plane z + 1 (and of the column two planes ahead)
-// are in flight while plane z is evaluated.  Undecided cells are queued
-// (at most one per thread and plane) and evaluated in float64 at the end by
-// consecutive threads.
+// z - 1, z and z + 1 and, as float64 inputs not yet converted, at z + 2, and
+// the halo threads the next plane's halo inputs, so that these loads are in
+// flight while a plane is evaluated (converting them where they are loaded
+// waited for memory once a plane).  Bound by issue and load latency, not by
+// memory: 256^3, sigma = B^2/rho, 566 MB, 224 -> 196 us with the inputs in flight,
+// the shorter conversion (f32_mag) and the residual-corrected quotient, six
+// resident blocks for that kind (five: 206).
+// Undecided cells are queued (at most one per thread and plane) and evaluated
+// in float64 at the end by consecutive threads.
 template <int KIND>
-__global__ void __launch_bounds__(TAG_TILE) k_tag_tile(TagArgs a)
+__global__ void __launch_bounds__(TAG_TILE, KIND == 2 ? 6 : 5) k_tag_tile(TagArgs a)
 {
     __shared__ float s[2][TAG_TY + 2][TAG_TX + 2];
     __shared__ unsigned q[TAG_SZ * TAG_TILE];
@@ -239,7 +286,7 @@ __global__ void __launch_bounds__(TAG_TILE) k_tag_tile(TagArgs a)
     const int tx = rel % ntx, ty = (rel / ntx) % nty, sz = rel / (ntx * nty);
     const int lx = threadIdx.x % TAG_TX, ly = threadIdx.x / TAG_TX;
     const int x = tx * TAG_TX + lx, y = ty * TAG_TY + ly;
-    const int z0 = sz * TAG_SZ, z1 = min(z0 + TAG_SZ, P.n[2]);
+    const int z0 = sz * a.sz, z1 = min(z0 + a.sz, P.n[2]);
     const bool z3 = a.ndim > 2;
     const int g2 = z3 ? AMR_NG : 0;
     const long long N0 = P.n[0] + 2 * AMR_NG, N1 = P.n[1] + 2 * AMR_NG, PS = N0 * N1;
@@ -269,19 +316,22 @@ __global__ void __launch_bounds__(TAG_TILE) k_tag_tile(TagArgs a)
         hoff = P.base + (long long)(gy + AMR_NG) * N0 + (gx + AMR_NG) + (long long)g2 * PS;
     }
     if (threadIdx.x == 0) qn = 0;
-    float prev = 0.0f, cur = 0.0f, nxt = 0.0f, nn = 0.0f, hv = 0.0f;
+    // float64 inputs in flight: the own column's of plane z + 2, the halo
+    // entry's of plane z + 1
+    float prev = 0.0f, cur = 0.0f, nxt = 0.0f;
+    TagRaw<KIND> own, hal;
+    const bool more = z0 + 1 < z1;
     if (own_ok) {
         cur = tag_sigma32<KIND>(a.U, a.us, col + (long long)z0 * PS);
         if (z3) {
             prev = tag_sigma32<KIND>(a.U, a.us, col + (long long)(z0 - 1) * PS);
             nxt = tag_sigma32<KIND>(a.U, a.us, col + (long long)(z0 + 1) * PS);
-            if (z0 + 1 < z1) nn = tag_sigma32<KIND>(a.U, a.us, col + (long long)(z0 + 2) * PS);
+            if (more) tag_load<KIND>(a.U, a.us, col + (long long)(z0 + 2) * PS, own);
         }
     }
-    if (hok) hv = tag_sigma32<KIND>(a.U, a.us, hoff + (long long)z0 * PS);
     s[0][ly + 1][lx + 1] = cur;
-    if (threadIdx.x < NH) s[0][hy][hx] = hv;
-    if (hok && z0 + 1 < z1) hv = tag_sigma32<KIND>(a.U, a.us, hoff + (long long)(z0 + 1) * PS);
+    if (threadIdx.x < NH) s[0][hy][hx] = hok ? tag_sigma32<KIND>(a.U, a.us, hoff + (long long)z0 * PS) : 0.0f;
+    if (hok && more) tag_load<KIND>(a.U, a.us, hoff + (long long)(z0 + 1) * PS, hal);
     __syncthreads();
     unsigned acc = 0;
     for (int z = z0; z < z1; ++z) {
@@ -305,12 +355,14 @@ __global__ void __launch_bounds__(TAG_TILE) k_tag_tile(TagArgs a)
         tag_count(tag, acc);
         if (z + 1 < z1) {
             s[b ^ 1][ly + 1][lx + 1] = nxt;
-            if (threadIdx.x < NH) s[b ^ 1][hy][hx] = hv;
-            if (hok && z + 2 < z1) hv = tag_sigma32<KIND>(a.U, a.us, hoff + (long long)(z + 2) * PS);
             prev = cur;
             cur = nxt;
-            nxt = nn;
-            if (own_ok && z + 2 < z1) nn = tag_sigma32<KIND>(a.U, a.us, col + (long long)(z + 3) * PS);
+            if (own_ok) nxt = tag_conv<KIND>(own);
+            if (threadIdx.x < NH) s[b ^ 1][hy][hx] = hok ? tag_conv<KIND>(hal) : 0.0f;
+            if (z + 2 < z1) {
+                if (own_ok) tag_load<KIND>(a.U, a.us, col + (long long)(z + 3) * PS, own);
+                if (hok) tag_load<KIND>(a.U, a.us, hoff + (long long)(z + 2) * PS, hal);
+            }
         }
         __syncthreads();
     }
