@@ -43,7 +43,10 @@ inline void group_widths(Group &G, int ndim, bool f64, bool mt)
 // serial chains.  With B blocks on S SMs, a step of the march takes a + k
 // while k blocks share an SM (a: the latency part, in units of the throughput
 // part of one block), at most `fit` of them, and the whole launch L times
-//   floor(B / (fit S)) (a + fit) + (a + ceil(rest / S), if a rest is left).
+//   floor(B / (fit S)) (a + fit) + (a + ceil(rest / S), if a rest is left),
+// L the batch's mean, and no less than its longest march takes (a level of 162
+// patches of 8^3 to 64^3 marched 64 cells without this, z and y 319 and 435 us;
+// 16 with it, 230 and 254).
 // Fitted on the GB300 to 11 lengths of 21 shapes: a = 1.5 in float32, 0.15 for
 // float64 MHD, whose single block per SM already fills the FP64 pipe; the
 // model picks the fastest or one within 4%.  us per step at the fixed 16 and at
@@ -72,7 +75,7 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int 
         for (int c : cand) {
             double t = 0.0;
             for (int D = 1; D < ndim; ++D) {
-                double blocks = 0.0, steps = 0.0;
+                double blocks = 0.0, steps = 0.0, longest = 0.0;
                 for (int i = 0; i < ng; ++i) {
                     const Group &G = g[i];
                     const int seg = ring || pick(G) ? c : G.seg, len = seg < G.n[D] ? seg : G.n[D];
@@ -80,11 +83,14 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int 
                                                              : Tiles::sweep_m(G.n, D, G.xw, seg));
                     blocks += b;
                     steps += b * (len + (ring ? 1 : 2));
+                    if (len + (ring ? 1 : 2) > longest) longest = len + (ring ? 1 : 2);
                 }
                 if (blocks <= 0.0) continue;
                 const double k = blocks / S, full = (double)(long long)(k / fit), rest = k - full * fit;
                 const double tail = rest > 1e-9 ? a + (double)(long long)(rest + 0.999999) : 0.0;
-                t += steps / blocks * (full * (a + fit) + tail + late);
+                const double mean = steps / blocks * (full * (a + fit) + tail + late);
+                const double chain = longest * (a + (k < fit ? (double)(long long)(k + 0.999999) : fit));
+                t += mean > chain ? mean : chain;
             }
             if (best == 0 || t < top) {
                 top = t;
