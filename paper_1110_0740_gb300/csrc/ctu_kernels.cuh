@@ -1644,7 +1644,7 @@ k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
     if (LAST) damp = patch_damp(a, P);
     unsigned int fl = 0;
     R mx = R(0);
-    if (STEP && !ok) x = o = 0;  // cells to point at; no iteration
+    if (STEP && !ok) x = o = 0;  // cells to point at; no copy, no iteration
     if (ok || STEP) {
         const int j0 = seg * SEGL, j1 = STEP && !ok ? j0 - 2 : min(j0 + SEGL, nD);
         const int st = dstr(P, D);
@@ -1744,7 +1744,7 @@ k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
                 }
                 cp_async_commit();
             };
-            issue(j0 - 1, c, (j0 - 1) & 1);
+            if (!STEP || ok) issue(j0 - 1, c, (j0 - 1) & 1);  // an idle thread would not wait for its copies
             for (int j = j0 - 1; j <= (STEP ? j0 + SEGL : j1); ++j, c += st) {
                 if constexpr (STEP) {
                     __syncthreads();
