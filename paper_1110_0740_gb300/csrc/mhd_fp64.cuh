@@ -48,11 +48,25 @@ __device__ __forceinline__ long long d_mag(double x) { return d_bits(x) & ~D_SIG
 __device__ __forceinline__ long long d_twice(long long m) { return m >= D_ONE_EXP ? m + D_ONE_EXP : m << 1; }
 __device__ __forceinline__ long long d_halve(long long m) { return m >= 2 * D_ONE_EXP ? m - D_ONE_EXP : m >> 1; }
 
-// 1/x: seed r and residual e = 1 - x r, r (1 + e + e^2).
-__device__ __forceinline__ double d_rcp64(double x)
+#ifdef __CUDACC__  // the hardware's seeds (a host build brings its own)
+__device__ __forceinline__ double d_rcp_seed(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+__device__ __forceinline__ double d_rsqrt_seed(double x)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+#endif
+
+// 1/x: seed r and residual e = 1 - x r, r (1 + e + e^2).
+__device__ __forceinline__ double d_rcp64(double x)
+{
+    const double r = d_rcp_seed(x);
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
@@ -60,8 +74,7 @@ __device__ __forceinline__ double d_rcp64(double x)
 // y (1 + e/2 + 3 e^2/8).  x below the normal range: y = 0, s = 0.
 __device__ __forceinline__ void d_roots64(double x, double &y, double &s)
 {
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double y0 = d_rsqrt_seed(x);
     const double p = x * y0;
     const double e = fma(-p, y0, 1.0);
     const double t = fma(e, 0.375, 0.5) * e;

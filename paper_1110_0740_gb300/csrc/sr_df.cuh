@@ -764,7 +764,9 @@ struct SrOut64 {
 // Gamma; the Taub-Mathews gas, gam = 0, keeps sr_prim64): W from sr_seed on the
 // FP32 pipe, so that one float64 evaluation of the energy equation remains,
 // with v^2 and p carried over its step by their first-order terms (a step of at
-// most 1e-9 W: a remainder of 1e-18).  sr_prim64 took several evaluations from
+// most 1e-9 W that moves 1 - v^2 by at most 7.5e-9 of itself: remainders of 1e-18
+// W (1 - v^2) and 1e-17 rho; the step alone moves 1 - v^2 by up to 2e-9 gamma^2 of
+// itself, and p came out 1e-4 off at gamma = 1000).  sr_prim64 took several evaluations from
 // a guess, and its bracketed iteration tens of them for the lanes without a
 // usable one, the whole warp waiting.  64^3 beam, ms per launch before and
 // after (with the FP64 forms of the fluxes): prim 1.29 and 0.095, sweep z 7.5 and
@@ -807,9 +809,11 @@ static __device__ __noinline__ SrOut64 sr_prim_fp64(SrCons c, double gam, double
             const double dF = (1.0 - dp) + fma(0.5 * B2, dv2, t2W);
             const double dW = -f * d_rcp64(dF), Wn = W + dW;
             if (!d_pos(Wn)) break;
-            if (d_mag(dW) <= d_mag(1.0e-9 * W)) {
-                const double evn = fma(-dv2, dW, ev), pn = fma(dp, dW, p);
-                if (!d_pos(evn)) break;
+            const double evn = fma(-dv2, dW, ev);
+            // in units of ev's last place; far off for evn <= 0 and for nans
+            const unsigned long long moved = (unsigned long long)d_bits(evn) - (unsigned long long)d_bits(ev);
+            if (d_mag(dW) <= d_mag(1.0e-9 * W) && moved + (1ull << 25) <= 2ull << 25) {
+                const double pn = fma(dp, dW, p);
                 const double iq = d_rcp64(Wn + B2), SW = S * d_rcp64(Wn);
                 o.V[0] = D * d_sqrt64(evn);
 #pragma unroll

@@ -31,3 +31,16 @@ inline float __uint_as_float(unsigned u) { return bits_as<float>(u); }
 inline unsigned __float_as_uint(float f) { return bits_as<unsigned>(f); }
 inline long long __double_as_longlong(double d) { return bits_as<long long>(d); }
 inline double __longlong_as_double(long long u) { return bits_as<double>(u); }
+// float64 seeds like the hardware's approximations: about 2^-23 and 2^-22 off,
+// results and arguments below the normal range zero
+namespace ctu {
+inline double seed_off(double r, double rel)
+{
+    const uint64_t h = bits_as<uint64_t>(r) * 0x9E3779B97F4A7C15ull;
+    r *= 1.0 + rel * ((double)(h >> 40) / 8388608.0 - 1.0);
+    return std::fabs(r) < 2.2250738585072014e-308 ? std::copysign(0.0, r) : r;
+}
+inline double seed_arg(double x) { return std::fabs(x) < 2.2250738585072014e-308 ? std::copysign(0.0, x) : x; }
+inline double d_rcp_seed(double x) { return seed_off(1.0 / seed_arg(x), 1.19e-7); }
+inline double d_rsqrt_seed(double x) { return seed_off(1.0 / std::sqrt(seed_arg(x)), 2.38e-7); }
+} // namespace ctu
