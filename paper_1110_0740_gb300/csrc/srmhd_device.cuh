@@ -224,15 +224,32 @@ __device__ __forceinline__ unsigned int sr_prim_tail(const double (&U)[NV], doub
     return st;
 }
 
-// V(U) in float64.  With a guess W0 > 0 (the W of a nearby state) plain
-// Newton steps are tried first (at most 12); if one leaves the physical
+// The recovery in units of the state's own: the energy equation's products reach
+// W^4 in float64 (their reciprocals start from float32 seeds) and W^7 in float32,
+// so that states of tau below 1e-10 or above 1e9 left float32's range and came out
+// wrong with status 0.  A state whose tau = E + D lies outside [2^-10, 2^11) is
+// scaled by powers of two (D, m, E by 2^(-2h), B by 2^-h, tau into [1, 4)), which
+// rounds nothing, and rho and p are scaled back.
+__device__ __forceinline__ double sr_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+// h for tau = 2^e (1 + ...)
+__device__ __forceinline__ int sr_half_exp(int e)
+{
+    return e >= -10 && e <= 10 ? 0 : (e < -1020 ? -1020 : e > 1020 ? 1020 : e) >> 1;
+}
+__device__ __forceinline__ int sr_unit(double tau)
+{
+    const int hw = __double2hiint(tau);  // positive and normal, or not scaled
+    return hw >= 1 << 20 && hw < 0x7FF << 20 ? sr_half_exp((hw >> 20) - 1023) : 0;
+}
+
+// V(U) in float64, U in its own units.  With a guess W0 > 0 (the W of a
+// nearby state) plain Newton steps are tried first (at most 12); if one leaves the physical
 // range or does not converge, and always without a guess, the bracketed
 // iteration runs: [Wlo, Whi] with f(Whi) > 0 found by doubling from tau,
 // Newton steps outside the bracket replaced by bisection.  Bounded: at most
 // 64 doublings and 100 iterations.  Returns status bits (0, ST_REC for no
 // convergence, ST_NEG / ST_SUPER).
-__device__ __forceinline__ unsigned int sr_prim64(const double (&U)[NV], double gam, double (&V)[NV],
-                                                  double W0 = 0.0)
+__device__ __forceinline__ unsigned int sr_prim64_u(const double (&U)[NV], double gam, double (&V)[NV], double W0)
 {
     const double D = U[0], tau = U[4] + U[0];
     const double m2 = U[1] * U[1] + U[2] * U[2] + U[3] * U[3];
@@ -293,18 +310,17 @@ __device__ __forceinline__ unsigned int sr_prim64(const double (&U)[NV], double 
     return sr_prim_tail(U, W, v2, p, S, B2, D, conv, phys, V);
 }
 
-// V(U) for the mixed path.  Newton steps in float32 from the guess W0 (else
-// tau - B^2/2) bring W near float accuracy on the FP32 pipe; then float64
+// V(U) for the mixed path, U in its own units.  Newton steps in float32 from
+// the guess W0 (else tau - B^2/2) bring W near float accuracy on the FP32 pipe; then float64
 // Newton steps on the float64 energy equation follow (at most three), each
 // squaring the relative error: once a step moves W by at most 1e-5 W the
 // error left is of order 1e-10 relative, below the float32 rounding of the
 // mixed path's fluxes.  v^2 and p are carried from that evaluation to the
 // final W by their first-order Taylor terms (remainder of the order of the
 // step squared).  A non-physical iterate, or no acceptance within the three
-// steps, hands over to the bracketed float64 iteration of sr_prim64.  Float64
+// steps, hands over to the bracketed float64 iteration of sr_prim64_u.  Float64
 // inputs are rounded to float by integer operations (df_split).
-__device__ __forceinline__ unsigned int sr_prim_mixed(const double (&U)[NV], double gam, double (&V)[NV],
-                                                      double W0 = 0.0)
+__device__ __forceinline__ unsigned int sr_prim_mixed_u(const double (&U)[NV], double gam, double (&V)[NV], double W0)
 {
     const double D = U[0], tau = U[4] + U[0];
     const double m2 = U[1] * U[1] + U[2] * U[2] + U[3] * U[3];
@@ -312,20 +328,20 @@ __device__ __forceinline__ unsigned int sr_prim_mixed(const double (&U)[NV], dou
     const double S = U[1] * U[5] + U[2] * U[6] + U[3] * U[7];
     const double S2 = S * S;
     const double g1 = gam > 0.0 ? (gam - 1.0) * rcp64(gam) : 0.0;
-    if (!(D > 0.0) || !(tau > 0.0)) return sr_prim64(U, gam, V, W0);
+    if (!(D > 0.0) || !(tau > 0.0)) return sr_prim64_u(U, gam, V, W0);
     auto tof = [](double x) {
         const df h = df_split(x);
         return h.hi + h.lo;
     };
     const float Df = tof(D), tauf = tof(tau), m2f = tof(m2), B2f = tof(B2), S2f = tof(S2), g1f = tof(g1);
     if (!(W0 > 0.0)) W0 = tau - 0.5 * B2;
-    if (!(W0 > 0.0)) return sr_prim64(U, gam, V, 0.0);
+    if (!(W0 > 0.0)) return sr_prim64_u(U, gam, V, 0.0);
     float Wf = tof(W0);
     for (int it = 0; it < 12; ++it) {
         float f, dfw;
-        if (!sr_energy_f(Wf, Df, m2f, S2f, B2f, tauf, g1f, f, dfw)) return sr_prim64(U, gam, V, W0);
+        if (!sr_energy_f(Wf, Df, m2f, S2f, B2f, tauf, g1f, f, dfw)) return sr_prim64_u(U, gam, V, W0);
         const float Wn = Wf - f / dfw;
-        if (!(Wn > 0.0f)) return sr_prim64(U, gam, V, W0);
+        if (!(Wn > 0.0f)) return sr_prim64_u(U, gam, V, W0);
         const bool done = fabsf(Wn - Wf) <= 2.0e-6f * Wf;
         Wf = Wn;
         if (done) break;
@@ -345,7 +361,51 @@ __device__ __forceinline__ unsigned int sr_prim_mixed(const double (&U)[NV], dou
         }
         W = Wn;
     }
-    return sr_prim64(U, gam, V, W);
+    return sr_prim64_u(U, gam, V, W);
+}
+
+// The same for a state in any units.  The scaled copy is out of line: inline it
+// cost the Taub-Mathews sweeps 1 to 3% on states that need none.
+struct SrScaled {
+    double V[NV];
+    unsigned int st;
+};
+template <bool MIXED>
+static __device__ __noinline__ SrScaled sr_prim_scaled(SrScaled U, int h, double gam, double W0)
+{
+    const double s2 = sr_pow2(-2 * h), s1 = sr_pow2(-h);
+    double X[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) X[q] = U.V[q] * (q < 5 ? s2 : s1);
+    SrScaled o;
+    o.st = MIXED ? sr_prim_mixed_u(X, gam, o.V, W0 * s2) : sr_prim64_u(X, gam, o.V, W0 * s2);
+    o.V[0] *= sr_pow2(2 * h);
+    o.V[4] *= sr_pow2(2 * h);
+#pragma unroll
+    for (int q = 5; q < NV; ++q) o.V[q] = U.V[q];
+    return o;
+}
+template <bool MIXED>
+__device__ __forceinline__ unsigned int sr_prim_units(const double (&U)[NV], double gam, double (&V)[NV], double W0)
+{
+    const int h = sr_unit(U[4] + U[0]);
+    if (h == 0) return MIXED ? sr_prim_mixed_u(U, gam, V, W0) : sr_prim64_u(U, gam, V, W0);
+    SrScaled o;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) o.V[q] = U[q];
+    o = sr_prim_scaled<MIXED>(o, h, gam, W0);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) V[q] = o.V[q];
+    return o.st;
+}
+__device__ __forceinline__ unsigned int sr_prim64(const double (&U)[NV], double gam, double (&V)[NV], double W0 = 0.0)
+{
+    return sr_prim_units<false>(U, gam, V, W0);
+}
+__device__ __forceinline__ unsigned int sr_prim_mixed(const double (&U)[NV], double gam, double (&V)[NV],
+                                                      double W0 = 0.0)
+{
+    return sr_prim_units<true>(U, gam, V, W0);
 }
 
 // The recovery of the working precision: float64 throughout for R = double,
