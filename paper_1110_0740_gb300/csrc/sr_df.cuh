@@ -278,6 +278,11 @@ __device__ __forceinline__ float sr_bracket_f(float D, float m2, float S2, float
 // Out of line: the sweeps recover three or four states a cell, and the copies
 // inlined (about 1000 instructions each) overflowed the instruction cache
 // (x sweep 36.1 ms at 256^3 with 15 of 20 stall cycles on instruction fetch).
+// Undecided outside tau in [2^-16, 2^16), where the float64 iteration scales the
+// state (sr_half_exp): below, the low parts of m^2, B^2 and their products drop
+// under the normal range and flush to zero, which the bounds, relative ones, do not
+// see (from tau ~ 2^-18 down p came out up to 12 ulp off).  Scaling here, inline or
+// in a call, cost the sweeps 3 to 4% in spills and instruction fetch.
 struct SrRec {
     float V[5];
     bool ok;
@@ -292,7 +297,8 @@ __device__ __forceinline__ bool sr_recover_in(const SrState &u, float W0, df g1,
     B2 = d_norm(B2.hi, B2.lo);
     S = d_norm(S.hi, S.lo);
     const float Sa = fabsf(sx.hi) + fabsf(sy.hi) + fabsf(sz.hi);
-    if (!(u.D.hi > 0.0f) || !(u.tau.hi > 0.0f)) return false;
+    // (D: the low part of rho needs 2^-126)
+    if (!(u.D.hi >= 8.8817841970012523e-16f) || !(u.tau.hi >= 1.52587890625e-5f && u.tau.hi < 65536.0f)) return false;
     if (!(W0 > 0.0f)) W0 = d_add(u.tau, d_neg(d_half(B2))).hi;
     if (!(W0 > 0.0f)) return false;
     // float32 Newton, as sr_prim_mixed; a two-cycle (the float32 residual's

@@ -227,14 +227,14 @@ __device__ __forceinline__ unsigned int sr_prim_tail(const double (&U)[NV], doub
 // The recovery in units of the state's own: the energy equation's products reach
 // W^4 in float64 (their reciprocals start from float32 seeds) and W^7 in float32,
 // so that states of tau below 1e-10 or above 1e9 left float32's range and came out
-// wrong with status 0.  A state whose tau = E + D lies outside [2^-10, 2^11) is
+// wrong with status 0.  A state whose tau = E + D lies outside [2^-16, 2^16) is
 // scaled by powers of two (D, m, E by 2^(-2h), B by 2^-h, tau into [1, 4)), which
 // rounds nothing, and rho and p are scaled back.
 __device__ __forceinline__ double sr_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 // h for tau = 2^e (1 + ...)
 __device__ __forceinline__ int sr_half_exp(int e)
 {
-    return e >= -10 && e <= 10 ? 0 : (e < -1020 ? -1020 : e > 1020 ? 1020 : e) >> 1;
+    return e >= -16 && e <= 15 ? 0 : (e < -1020 ? -1020 : e > 1020 ? 1020 : e) >> 1;
 }
 __device__ __forceinline__ int sr_unit(double tau)
 {

@@ -15,8 +15,21 @@ using std::isfinite;
 inline float __fadd_rn(float a, float b) { return a + b; }
 inline float __fmul_rn(float a, float b) { return a * b; }
 inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
-inline float __fdividef(float a, float b) { return a / b; }
-inline float rsqrtf(float x) { return (float)(1.0 / std::sqrt((double)x)); }
+#ifdef SEED_ULPS  // the approximate forms, up to that many units in the last place off
+inline float ulps_off(float r)
+{
+    uint32_t u;
+    std::memcpy(&u, &r, 4);
+    if ((u & 0x7F800000u) == 0u || (u & 0x7F800000u) == 0x7F800000u) return r;
+    u += (u * 0x9E3779B9u >> 16) % (2 * SEED_ULPS + 1) - SEED_ULPS;
+    std::memcpy(&r, &u, 4);
+    return r;
+}
+#else
+inline float ulps_off(float r) { return r; }
+#endif
+inline float __fdividef(float a, float b) { return ulps_off(a / b); }
+inline float rsqrtf(float x) { return ulps_off((float)(1.0 / std::sqrt((double)x))); }
 template <class T, class F> inline T bits_as(F f)
 {
     T t;
