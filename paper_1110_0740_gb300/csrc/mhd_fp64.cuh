@@ -35,14 +35,14 @@ namespace ctu {
 
 __device__ __forceinline__ long long d_bits(double x) { return __double_as_longlong(x); }
 __device__ __forceinline__ double d_from(long long b) { return __longlong_as_double(b); }
-constexpr long long D_SIGN = (long long)0x8000000000000000ull, D_ONE_EXP = 1ll << 52;
+constexpr long long D_SIGN = (long long)0x8000000000000000ull, D_ONE_EXP = 1ll << 52, D_INF = 0x7FFll << 52;
 
-// x > 0 (also +inf), false for zeros and nans; x >= 0 of a number
+// x > 0 (also +inf) and x >= 0, false for nans, whose sign bit says nothing
 __device__ __forceinline__ bool d_pos(double x)
 {
     return (unsigned long long)(d_bits(x) - 1) < 0x7FF0000000000000ull;
 }
-__device__ __forceinline__ bool d_nonneg(double x) { return d_bits(x) >= 0 || d_bits(x) == D_SIGN; }
+__device__ __forceinline__ bool d_nonneg(double x) { return (unsigned long long)d_bits(x) <= (unsigned long long)D_INF || d_bits(x) == D_SIGN; }
 // |x| as an ordered integer, twice a magnitude, half of it
 __device__ __forceinline__ long long d_mag(double x) { return d_bits(x) & ~D_SIGN; }
 __device__ __forceinline__ long long d_twice(long long m) { return m >= D_ONE_EXP ? m + D_ONE_EXP : m << 1; }
@@ -90,12 +90,12 @@ __device__ __forceinline__ double d_sqrt64(double x)
 }
 
 // Monotonised-central slope of dm, dp (mc_slope) as a bit pattern: sign times
-// min(|dm + dp|/2, 2|dm|, 2|dp|), 0 unless both have one sign.
+// min(|dm + dp|/2, 2|dm|, 2|dp|), 0 unless both have one sign and neither is a nan.
 __device__ __forceinline__ double d_mc64(double dm, double dp)
 {
     const long long am = d_mag(dm), ap = d_mag(dp);
-    const long long t = d_twice(am < ap ? am : ap), h = d_halve(d_mag(dm + dp));
-    const bool same = (d_bits(dm) ^ d_bits(dp)) >= 0 && am != 0 && ap != 0;
+    const long long a = am < ap ? am : ap, b = d_mag(dm + dp), t = d_twice(a), h = d_halve(b);
+    const bool same = (d_bits(dm) ^ d_bits(dp)) >= 0 && a != 0 && b <= D_INF;
     return same ? d_from((h < t ? h : t) | (d_bits(dm) & D_SIGN)) : 0.0;
 }
 
@@ -107,7 +107,7 @@ __device__ __forceinline__ void d_reconstruct64(const double (&d)[4], int lim, d
 {
     if (recon_hybrid(RK) && lim == 2) {
         const long long am = d_mag(d[1]), ap = d_mag(d[2]);
-        const bool same = (d_bits(d[1]) ^ d_bits(d[2])) >= 0 && am != 0 && ap != 0;
+        const bool same = (d_bits(d[1]) ^ d_bits(d[2])) >= 0 && am != 0 && ap != 0 && am <= D_INF && ap <= D_INF;
         const double s = same ? d_from(d_halve(am < ap ? am : ap) | (d_bits(d[1]) & D_SIGN)) : 0.0;
         wp = s;
         wm = -s;
@@ -123,10 +123,11 @@ __device__ __forceinline__ void d_reconstruct64(const double (&d)[4], int lim, d
     const double p = fma(0.5, d[2], (s0 - sp) * (1.0 / 6.0));
     const double m = fma(-0.5, d[1], (sm - s0) * (1.0 / 6.0));
     const long long ap = d_mag(p), am = d_mag(m);
-    const bool extremum = (d_bits(p) ^ d_bits(m)) >= 0 && ap != 0 && am != 0;
+    const bool num = ap < D_INF && am < D_INF;  // a nan or an infinity stays one
+    const bool extremum = num && (d_bits(p) ^ d_bits(m)) >= 0 && ap != 0 && am != 0;
     const long long tp = d_twice(ap), tm = d_twice(am);
-    const double np = ap >= tm ? d_from(tm | (~d_bits(m) & D_SIGN)) : p;
-    const double nm = am >= tp ? d_from(tp | (~d_bits(p) & D_SIGN)) : m;
+    const double np = num && ap >= tm ? d_from(tm | (~d_bits(m) & D_SIGN)) : p;
+    const double nm = num && am >= tp ? d_from(tp | (~d_bits(p) & D_SIGN)) : m;
     wp = extremum ? 0.0 : np;
     wm = extremum ? 0.0 : nm;
 }
@@ -238,8 +239,16 @@ __device__ __forceinline__ void char_predict64(const double (&vs)[5][NV], double
     const double hps = 0.5 * h * ch * (dgp - dgm);
     const double vB = u * Bn + v1c * B1c + v2c * B2c;
     const double hr = hB * irho;
-    const double s[NV] = {vs[2][0], fma(Bn, hr, u), fma(B1c, hr, v1c), fma(B2c, hr, v2c),
-                          fma(gam - 1.0, Bn * hps - vB * hB, pc), Bn, fma(v1c, hB, B1c), fma(v2c, hB, B2c), vs[2][8]};
+    double s[NV] = {vs[2][0], fma(Bn, hr, u), fma(B1c, hr, v1c), fma(B2c, hr, v2c),
+                    fma(gam - 1.0, Bn * hps - vB * hB, pc), Bn, fma(v1c, hB, B1c), fma(v2c, hB, B2c), vs[2][8]};
+    // A nan or infinity in the cell itself makes both states nans whole, as it would
+    // as a term of every characteristic variable: the limiters drop its differences.
+    int top = 0;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) top = max(top, __double2hiint(vs[2][q]) & 0x7FFFFFFF);
+    const long long lost = top >= 0x7FF00000 ? 0x7FF8ll << 48 : 0ll;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) s[q] = d_from(d_bits(s[q]) | lost);
 
     // recombination with the right eigenvectors, added to the cell's state
     const double i2a2 = 0.5 * ia2, hrho = 0.5 * rho;

@@ -1,6 +1,7 @@
 // Host stand-ins for the CUDA names the relativistic recovery's headers use, so
 // that its arithmetic can be compiled and checked by the host compiler.
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -12,6 +13,8 @@ using std::fabs;
 using std::fmax;
 using std::fmin;
 using std::isfinite;
+using std::max;
+using std::min;
 inline float __fadd_rn(float a, float b) { return a + b; }
 inline float __fmul_rn(float a, float b) { return a * b; }
 inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
