@@ -372,12 +372,14 @@ ctu_status ctu_flux_registers(ctu_ctx *ctx, double *reg, const ctu_flux_window *
                               int nwin);
 
 /* Tile autotuner (launch configuration only; the paper has no counterpart).
- * A launch covers every patch shape of the batch; per shape, the kernels use
- * a thread-tile width along x (8, 16 or 32 lanes) and a marching segment
- * length along y and z (4 to 64 cells).  ctu_autotune times ctu_step on the
- * caller's batch for each candidate pair of every shape in turn (largest
- * shapes first, the others held fixed), keeps the fastest, and stores the
- * choice per shape in the context for every later call.  The choice changes
+ * A launch covers every patch shape of the batch; per shape, the marching
+ * kernels use a thread-tile width along x (8, 16 or 32 lanes) and a marching
+ * segment length along y and z, by default one that suits the whole batch (1
+ * to 64 cells).  ctu_autotune times ctu_step on the caller's batch as it runs
+ * by default, then for each candidate pair (segments of 4 to 64 cells) of every
+ * shape in turn (largest shapes first, the others held fixed), and stores the
+ * fastest per shape in the context for every later call, where one beats the
+ * default; the default stays otherwise.  The choice changes
  * only how cells map to threads: each cell's arithmetic, and so the result,
  * is the same for every choice.  U_out is overwritten (U_in is read only);
  * the bound flux registers are left untouched; d_dt_ch is read as in

@@ -800,6 +800,21 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         ms = best;
         return CTU_OK;
     };
+    // What an untuned step takes comes first (choose_segments; shapes tuned before
+    // start afresh): a shape is pinned only by a pair that beats it by 2%, more than
+    // two timings differ by, and the pins together only if their step is no slower.
+    // The candidates alone made small batches slower, since the rule takes segments
+    // down to one cell: 2-D 128^2 float64 177 us untuned and 264 tuned, 32^3 567 and
+    // 721.
+    auto afresh = [&]() -> ctu_status {
+        ctx->hpatch.clear();
+        return bind_patches(ctx, patches, npatch, s);
+    };
+    std::vector<std::array<int, 3>> pinned;
+    for (const Group &G : ctx->groups) ctx->tune.erase(shape_key(G.n));
+    st = afresh();
+    float rule = 0.0f;
+    if (st == CTU_OK) st = timed(rule);
     // coordinate descent over the shapes, largest first: for each, every
     // (tile width, segment) candidate with the other shapes fixed
     static const int kXw[] = {8, 16, 32};
@@ -807,29 +822,49 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
     for (size_t g = 0; g < ctx->groups.size() && st == CTU_OK; ++g) {
         Group &G = ctx->groups[g];
         int bx = G.xw, bs = G.seg;
-        float bt = 1e30f;
+        float bt = 0.0f;
+        bool beaten = false;
+        st = timed(bt);
+        bt *= 0.98f;
         const int nmax = std::max(G.n[0], std::max(G.n[1], G.n[2]));
         for (int xw : kXw) {
             if (xw > 8 && xw / 2 >= G.n[0] + 2) continue;  // wider than the patch
             for (int sg : kSeg) {
+                if (st != CTU_OK) break;
                 if (sg > 4 && sg / 2 >= nmax) continue;    // longer than any pencil
+                const int x0 = G.xw, s0 = G.seg;
                 G.xw = xw;
                 G.seg = sg;
-                if (!grid_fits(ctx->groups, ctx->cfg.ndim)) continue;
+                if (!grid_fits(ctx->groups, ctx->cfg.ndim)) {
+                    G.xw = x0;
+                    G.seg = s0;
+                    continue;
+                }
                 float t = 0.0f;
                 st = timed(t);
-                if (st != CTU_OK) break;
-                if (t < bt) {
+                if (st == CTU_OK && t < bt) {
                     bt = t;
                     bx = xw;
                     bs = sg;
+                    beaten = true;
                 }
             }
-            if (st != CTU_OK) break;
         }
         G.xw = bx;
         G.seg = bs;
-        ctx->tune[shape_key(G.n)] = {bx, bs};
+        if (beaten) {
+            ctx->tune[shape_key(G.n)] = {bx, bs};
+            pinned.push_back(shape_key(G.n));
+        }
+    }
+    if (st == CTU_OK && !pinned.empty()) {
+        float t = 0.0f;
+        st = afresh();
+        if (st == CTU_OK) st = timed(t);
+        if (st == CTU_OK && t > rule) {
+            for (const auto &k : pinned) ctx->tune.erase(k);
+            st = afresh();
+        }
     }
     ctx->tuning = false;
     cudaEventDestroy(e0);
