@@ -379,7 +379,7 @@ ctu_status ctu_flux_registers(ctu_ctx *ctx, double *reg, const ctu_flux_window *
  * by default, then for each candidate pair (segments of 4 to 64 cells) of every
  * shape in turn (largest shapes first, the others held fixed), and stores the
  * fastest per shape in the context for every later call, where one beats the
- * default; the default stays otherwise.  The choice changes
+ * default or is its own; the default stays otherwise.  The choice changes
  * only how cells map to threads: each cell's arithmetic, and so the result,
  * is the same for every choice.  U_out is overwritten (U_in is read only);
  * the bound flux registers are left untouched; d_dt_ch is read as in
@@ -389,10 +389,14 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
                         const ctu_patch *patches, int npatch, const double *d_dt_ch,
                         void *stream);
 
-/* The tile width *xw and segment length *seg the context uses for patches of
- * interior shape n[3] (autotuned if ctu_autotune saw that shape, else the
- * default rule: 32 lanes for n[0] >= 24, 16 for n[0] >= 12, else 8; 16
- * cells, which a step replaces by the length that suits the whole batch). */
+/* The tile width *xw and segment length *seg pinned for patches of interior
+ * shape n[3] by ctu_autotune; for a shape without a pin the default width (32
+ * lanes for n[0] >= 24, 16 for n[0] >= 12, else 8) and 16, the length a step
+ * starts from and replaces by the one, of 1 to 64 cells, that suits the whole
+ * batch.  The pair governs the marching sweeps along y and z (the width also
+ * the flags, speeds and cell-wise kernels); the x sweep, the first-order
+ * stage and the corner coupling along y and z take theirs from the shape and
+ * the batch. */
 ctu_status ctu_tile_params(ctu_ctx *ctx, const int n[3], int *xw, int *seg);
 
 /* ---- Level operators (Section 4 of Mignone et al. 2012; Cartesian) ------

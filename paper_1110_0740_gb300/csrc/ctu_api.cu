@@ -811,6 +811,7 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         return bind_patches(ctx, patches, npatch, s);
     };
     std::vector<std::array<int, 3>> pinned;
+    bool other = false;  // a pin that is not the default's own pair
     for (const Group &G : ctx->groups) ctx->tune.erase(shape_key(G.n));
     st = afresh();
     float rule = 0.0f;
@@ -852,12 +853,15 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         }
         G.xw = bx;
         G.seg = bs;
-        if (beaten) {
+        // the default's own pair, if it is one of the candidates, is kept as such: what
+        // ctu_tile_params reports of a tuned shape then is what runs
+        if (beaten || std::find(std::begin(kSeg), std::end(kSeg), bs) != std::end(kSeg)) {
             ctx->tune[shape_key(G.n)] = {bx, bs};
             pinned.push_back(shape_key(G.n));
+            other |= beaten;
         }
     }
-    if (st == CTU_OK && !pinned.empty()) {
+    if (st == CTU_OK && other) {
         float t = 0.0f;
         st = afresh();
         if (st == CTU_OK) st = timed(t);

@@ -277,7 +277,8 @@ def ctu_autotune(ctx, U_in, U_out, stride, patches, d_dt_ch, stream=None):
 
 
 def ctu_tile_params(ctx, n):
-    """(tile width along x, marching segment) used for interior shape n."""
+    """(tile width along x, marching segment) pinned for interior shape n by
+    ctu_autotune, else the defaults (see include/ctu.h)."""
     arr = (ctypes.c_int * 3)(*[int(v) for v in n])
     xw, seg = ctypes.c_int(), ctypes.c_int()
     _check(_lib().ctu_tile_params(ctx, arr, ctypes.byref(xw), ctypes.byref(seg)), "ctu_tile_params")
