@@ -24,6 +24,15 @@ def prog(tmp_path_factory):
 def test_a_nan_stays_one(prog):
     """No flux and no predicted value is a number where the generic functions,
     whose comparisons a nan fails, give a nan."""
-    lost, both = map(int, subprocess.run([prog], check=True, capture_output=True, text=True).stdout.split())
+    lost, both = map(int, subprocess.run([prog, "nan"], check=True, capture_output=True, text=True).stdout.split())
     assert both > 100000
     assert lost == 0
+
+
+def test_no_less_accurate_than_ieee_forms(prog):
+    """Against long double, on 200000 random states from nearly uniform to rough:
+    the predicted states (MC, PPM) and the HLLD fluxes are no further off than the
+    generic functions' in IEEE double."""
+    out = subprocess.run([prog, "err", "200000", "1"], check=True, capture_output=True, text=True).stdout
+    for ieee, here in (map(float, line.split()) for line in out.splitlines()):
+        assert 0.0 < here <= ieee
