@@ -319,7 +319,7 @@ static ctu_status bind_patches(ctu_ctx *ctx, const ctu_patch *p, int np, cudaStr
     if (!grid_fits(g2, ctx->cfg.ndim)) return CTU_EINVAL;
     std::vector<Group> g3(g2);
     choose_segments(g3.data(), (int)g3.size(), ctx->cfg.ndim, ctx->cfg.precision == CTU_FP64,
-                    ctx->cfg.physics == CTU_SRMHD, ctx->sms,
+                    ctx->cfg.physics == CTU_SRMHD, ctx->cfg.eos == CTU_EOS_TM, ctx->sms,
                     [&](const Group &G) { return ctx->tune.find(shape_key(G.n)) == ctx->tune.end(); });
     if (grid_fits(g3, ctx->cfg.ndim)) g2.swap(g3);
     if (np > ctx->dpatch_cap) {

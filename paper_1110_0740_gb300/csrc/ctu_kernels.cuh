@@ -1608,8 +1608,13 @@ template <class R, int MODE> __host__ __device__ constexpr int sweep_m_smem()
 // BLOCK/xw (other-dimension, segment) pairs.  Float: the next cell's inputs
 // are staged in shared memory by cp.async (sweep_m_smem bytes per block);
 // double: they are prefetched into L1.
-template <int PHYS, class R, int PPM, int IFACE64, int D, int MODE>
-__global__ void __launch_bounds__(BLOCK, PHYS == PH_SR && sizeof(R) == 4 ? CTU_MARCH_MINB_SR : CTU_MARCH_MINB)
+// TM: the Taub-Mathews gas, whose recoveries are the float64 iterations: bound by the
+// FP64 pipe and by the lanes that iterate longest, it keeps three blocks an SM, no
+// barrier and the compiler's own sums (us a step of the beam, with the ideal gas's
+// barrier and four blocks and so: 64^3 6500 and 5740, 128^3 18630 and 17200, 200^3
+// 47100 and 47420).
+template <int PHYS, class R, int PPM, int IFACE64, int D, int MODE, bool TM = false>
+__global__ void __launch_bounds__(BLOCK, PHYS == PH_SR && sizeof(R) == 4 && !TM ? CTU_MARCH_MINB_SR : CTU_MARCH_MINB)
 k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
 {
     constexpr int O = D == 1 ? 2 : 1;  // the other transverse dimension
@@ -1633,7 +1638,7 @@ k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
     // that they fetch the recoveries' code (more than the instruction cache
     // holds at once) together: 256^3 beam, z and y 7.9 -> 7.16 and 7.09 ms.  Every
     // thread of the block runs the same number of iterations, idle ones empty.
-    constexpr bool STEP = PHYS == PH_SR && STAGED;
+    constexpr bool STEP = PHYS == PH_SR && STAGED && !TM;
     const R gam = pgam<R>(a), ch = pch<R>(a.sp);
     const R dtr = pdt<R>(a.sp);
     const double dtd = a.sp->dt;
@@ -1699,7 +1704,7 @@ k_sweep_m(StepArgs a, GroupTable gt, const R *Vs, const R *L1, R *A)
                 } else if constexpr (FIRST) {
 #pragma unroll
                     for (int q = 0; q < NV; ++q) A[q * a.sstride + cp] = s[q];
-                } else if constexpr (PHYS == PH_SR && sizeof(R) == 4) {  // fused, see sr_side
+                } else if constexpr (PHYS == PH_SR && sizeof(R) == 4 && !TM) {  // fused, see sr_side
 #pragma unroll
                     for (int q = 0; q < NV; ++q) A[q * a.sstride + cp] = __fmaf_rn(Fprev[q] - F[q], iD, Ap[q * as]);
                 } else {

@@ -99,9 +99,12 @@ template <class F> static void with_tm(int tm, F &&f)
 // Kernels that stage through more than the default 48 KB of dynamic shared
 // memory are opted in once per device (the carveout set to its maximum, so
 // that the register-limited number of blocks still fits).
-template <int PHYS, class R, int PPM, int IF64, int D, int MODE>
+template <int PHYS, class R, int PPM, int IF64, int D, int MODE, bool TM = false>
 static int launch_sweep_m(const StepArgs &a, const LaunchInfo &li, const R *Vs, const R *L1, R *A, cudaStream_t s)
 {
+    if constexpr (PHYS == PH_SR && sizeof(R) == 4 && !TM) {  // Taub-Mathews: kernels of its own
+        if (a.gam == 0.0) return launch_sweep_m<PHYS, R, PPM, IF64, D, MODE, true>(a, li, Vs, L1, A, s);
+    }
     constexpr int smem = sweep_m_smem<R, MODE>();
     if (smem > 48 * 1024) {
         static std::atomic<unsigned long long> done{0};
@@ -109,9 +112,9 @@ static int launch_sweep_m(const StepArgs &a, const LaunchInfo &li, const R *Vs, 
         cudaGetDevice(&dev);
         const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
         if (!(done.load() & bit) || !bit) {
-            cudaFuncSetAttribute(k_sweep_m<PHYS, R, PPM, IF64, D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem);
-            cudaFuncSetAttribute(k_sweep_m<PHYS, R, PPM, IF64, D, MODE>,
+            cudaFuncSetAttribute(k_sweep_m<PHYS, R, PPM, IF64, D, MODE, TM>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            cudaFuncSetAttribute(k_sweep_m<PHYS, R, PPM, IF64, D, MODE, TM>,
                                  cudaFuncAttributePreferredSharedMemoryCarveout, 100);
             done.fetch_or(bit);
         }
@@ -119,7 +122,7 @@ static int launch_sweep_m(const StepArgs &a, const LaunchInfo &li, const R *Vs, 
     return over_groups(
         li, [&](const Group &G) { return Tiles::sweep_m(G.n, D, G.xw, G.seg); },
         [&](const GroupTable &gt, unsigned nb) {
-            k_sweep_m<PHYS, R, PPM, IF64, D, MODE><<<nb, BLOCK, smem, s>>>(a, gt, Vs, L1, A);
+            k_sweep_m<PHYS, R, PPM, IF64, D, MODE, TM><<<nb, BLOCK, smem, s>>>(a, gt, Vs, L1, A);
         });
 }
 

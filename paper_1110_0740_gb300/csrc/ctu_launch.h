@@ -58,8 +58,12 @@ inline void group_widths(Group &G, int ndim, bool f64, bool mt)
 // fastest in float64, within 13% in float32 (6% on average).  us of the sweep along
 // z at 8 cells, at 16 and at the choice: 64^3 mixed 376, 580, 285; 128^3 mixed
 // 1103, 1036, 1036; 64^3 float64 1068, 1280, 1068.
+// The Taub-Mathews gas in float32 (float64 iterations, whose number differs most
+// between pencils): c = 2, fitted to 15 lengths of 14 boxes, within 9% of the fastest
+// (2% on average); us a step at c = 0.5 and 2: 48^3 5252 and 4219, 128^3 17390 and
+// 16440, 130 x 70 x 50 9390 and 8460.
 template <class Pick>
-inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int sms, Pick pick)
+inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, bool tm, int sms, Pick pick)
 {
     static const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
     const double S = sms > 0 ? sms : 152;
@@ -69,7 +73,7 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, int 
         // ones 128 (four), the float first-order ones about 95 (five)
         const double fit = f64 ? 3.0 : ring ? 5.0 : rel ? 4.0 : 3.0;
         const double a = rel && !ring ? (f64 ? 2.0 : 0.5) : f64 && !rel ? 0.15 : 1.5;
-        const double late = rel && !ring ? (f64 ? 0.75 : 0.5) : 0.0;
+        const double late = rel && !ring ? (f64 ? 0.75 : tm ? 2.0 : 0.5) : 0.0;
         int best = 0;
         double top = 0.0;
         for (int c : cand) {

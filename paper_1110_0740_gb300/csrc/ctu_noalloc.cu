@@ -202,7 +202,7 @@ extern "C" ctu_status ctu_step_noalloc(const ctu_config *cfg, const double *U_in
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
             li.sms = sms;
     }
-    choose_segments(groups, npatch, cfg->ndim, cfg->precision == CTU_FP64, false, li.sms,
+    choose_segments(groups, npatch, cfg->ndim, cfg->precision == CTU_FP64, false, false, li.sms,
                     [](const Group &) { return true; });
     if (cfg->precision == CTU_FP64)
         launch_step<double>(a, li, s);
