@@ -627,9 +627,11 @@ __device__ __forceinline__ float sr_w0_f(const double (&V)[NV], const StepArgs &
     return ev > 1.0e-6f ? w / ev : 0.0f;
 }
 
-// SRMHD interface state at n+1/2: U(V*) + T formed in float64, recovered by
-// the float64 Newton iteration (Eq. transv).
-template <class R, int D>
+// SRMHD interface state at n+1/2 (Eq. transv), V(U(V*) + T): mixed, formed and
+// recovered in double-float, by the float64 iteration where that leaves a lane
+// undecided and for the Taub-Mathews gas; FP64, formed in float64 and recovered by
+// sr_prim_fp64.
+template <class R>
 __device__ __forceinline__ unsigned int sr_interface(const R (&W)[NV], const R (&T)[NV], const StepArgs &a,
                                                      R (&out)[NV])
 {
@@ -717,8 +719,8 @@ __device__ __forceinline__ unsigned int trace_cell_t(const StepArgs &a, const De
         f |= interface_state<R, IFACE64>(pg, Tc, a, Vp);
         f |= interface_state<R, IFACE64>(mg, Tc, a, Vm);
     } else {
-        f |= sr_interface<R, D>(pg, Tc, a, Vp);
-        f |= sr_interface<R, D>(mg, Tc, a, Vm);
+        f |= sr_interface<R>(pg, Tc, a, Vp);
+        f |= sr_interface<R>(mg, Tc, a, Vm);
     }
     return f;
 }

@@ -11,9 +11,13 @@
 // 7.15 -> 0.95 ms, the sweeps along z, y, x 44.8 -> 6.7, 45.4 -> 6.7,
 // 56.1 -> 11.0 ms.  Only the five float32 values rho, v, p leave a recovery,
 // so double-float (~2^-46) decides their rounding for all but the few lanes
-// whose value lies within the arithmetic's error of a rounding boundary.  Those lanes, and every state that is not plainly physical, take
-// the float64 iteration instead (the callers' noinline slow paths), so that
-// every result is the float64 iteration's, bit for bit.
+// whose value lies within the arithmetic's error of a rounding boundary.  Those
+// lanes, every state that is not plainly physical, and those in units far from 1
+// (sr_recover_in) take the float64 iteration instead (the callers' noinline slow
+// paths).  The error bounds' constants come from trials, not from a proof (SR_K):
+// on the states tried the results are the float64 iteration's, rounded, bit for
+// bit, except for 3 values out of 2e6 decided states, at Lorentz factors near 1000
+// (two of them the nearer to a 113-bit solution, none further).
 //
 // The iterates follow sr_prim_mixed's: the same float32 Newton steps from the
 // same guess, then its float64 steps in double-float, with the first-order
@@ -74,11 +78,6 @@ __device__ __forceinline__ df d_mul(df x, df y)
 {
     const df p = d_two_prod(x.hi, y.hi);
     return d_norm(p.hi, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p.lo)));
-}
-__device__ __forceinline__ df d_mulf(df x, float y)
-{
-    const df p = d_two_prod(x.hi, y);
-    return d_norm(p.hi, __fmaf_rn(x.lo, y, p.lo));
 }
 __device__ __forceinline__ df d_sqr(df x)
 {
@@ -450,7 +449,7 @@ static __device__ __noinline__ SrOut sr_interface_slow(SrFace f, double gam)
 {
     double V[NV];
     SrOut o;
-    o.st = sr_interface64<float>(f.V, f.T, gam, V);
+    o.st = sr_interface64(f.V, f.T, gam, V);
 #pragma unroll
     for (int q = 0; q < NV; ++q) o.V[q] = (float)V[q];
     return o;
@@ -462,7 +461,7 @@ __device__ __forceinline__ SrOut sr_mh_slow_in(const SrCons &c, const SrFace &f,
 {
     double V[NV];
     SrOut o;
-    o.st = sr_mh_recover<float>(c.U, f.V, f.T, gam, V);
+    o.st = sr_mh_recover(c.U, f.V, f.T, gam, V);
 #pragma unroll
     for (int q = 0; q < NV; ++q) o.V[q] = (float)V[q];
     return o;

@@ -408,17 +408,6 @@ __device__ __forceinline__ unsigned int sr_prim_mixed(const double (&U)[NV], dou
     return sr_prim_units<true>(U, gam, V, W0);
 }
 
-// The recovery of the working precision: float64 throughout for R = double,
-// the mixed recovery for R = float.
-template <class R> __device__ __forceinline__ unsigned int sr_prim(const double (&U)[NV], double gam, double (&V)[NV],
-                                                                   double W0 = 0.0)
-{
-    if constexpr (sizeof(R) == 4)
-        return sr_prim_mixed(U, gam, V, W0);
-    else
-        return sr_prim64(U, gam, V, W0);
-}
-
 // Lower / upper signal speeds along the local normal (V[1] = v_n).
 template <class R>
 __device__ __forceinline__ void sr_speeds(const R (&V)[NV], R gam, R &lm, R &lp)
@@ -525,10 +514,9 @@ __device__ __forceinline__ void sr_mh_increment(const R (&vm1)[NV], const R (&v0
     for (int q = 0; q < NV; ++q) x[q] = h * (Fp[q] - Fm[q]);
 }
 
-// The half-step state V(U*), U* = U_i^n - x, in float64.  Newton starts from
-// the cell-centre W = w gamma^2 (U* is an O(dt) update of U_i).
-template <class R>
-__device__ __forceinline__ unsigned int sr_mh_recover(const double (&U0)[NV], const R (&v0)[NV], const R (&x)[NV],
+// The half-step state V(U*), U* = U_i^n - x, of the mixed path in float64.  Newton
+// starts from the cell-centre W = w gamma^2 (U* is an O(dt) update of U_i).
+__device__ __forceinline__ unsigned int sr_mh_recover(const double (&U0)[NV], const float (&v0)[NV], const float (&x)[NV],
                                                       double gamd, double (&Vs)[NV])
 {
     double Us[NV];
@@ -536,21 +524,21 @@ __device__ __forceinline__ unsigned int sr_mh_recover(const double (&U0)[NV], co
     for (int q = 0; q < NV; ++q) Us[q] = U0[q] - (double)x[q];
     const double v2c = (double)v0[1] * v0[1] + (double)v0[2] * v0[2] + (double)v0[3] * v0[3];
     const double Wc = sr_w<double>((double)v0[0], (double)v0[4], gamd) * rcp64(1.0 - v2c);
-    return sr_prim<R>(Us, gamd, Vs, Wc);
+    return sr_prim_mixed(Us, gamd, Vs, Wc);
 }
 
-// Interface state at n+1/2 in float64: V(U(W) + T), Newton from the W of the
-// predicted state (the transverse correction T is an O(dt) change).
-template <class R>
-__device__ __forceinline__ unsigned int sr_interface64(const R (&W)[NV], const R (&T)[NV], double gamd, double (&V)[NV])
+// Interface state at n+1/2 of the mixed path in float64: V(U(W) + T), Newton from
+// the W of the predicted state (the transverse correction T is an O(dt) change).
+__device__ __forceinline__ unsigned int sr_interface64(const float (&W)[NV], const float (&T)[NV], double gamd,
+                                                       double (&V)[NV])
 {
     double U[NV];
-    sr_cons<double, R>(W, gamd, U);
+    sr_cons<double, float>(W, gamd, U);
     const double v2 = (double)W[1] * W[1] + (double)W[2] * W[2] + (double)W[3] * W[3];
     const double W0 = sr_w<double>((double)W[0], (double)W[4], gamd) * rcp64(1.0 - v2);
 #pragma unroll
     for (int q = 0; q < NV; ++q) U[q] += (double)T[q];
-    return sr_prim<R>(U, gamd, V, W0);
+    return sr_prim_mixed(U, gamd, V, W0);
 }
 
 } // namespace ctu
