@@ -48,14 +48,17 @@ inline void group_widths(Group &G, int ndim, bool f64, bool mt)
 // patches of 8^3 to 64^3 marched 64 cells without this, z and y 319 and 435 us;
 // 16 with it, 230 and 254).
 // Fitted on the GB300 to 11 lengths of 21 shapes: a = 1.5 in float32, 0.15 for
-// float64 MHD, whose single block per SM already fills the FP64 pipe; the
-// model picks the fastest or one within 4%.  us per step at the fixed 16 and at
-// the model's choice: 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and 112,
-// 64^3 mixed 208 and 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
+// float64 MHD, whose single block per SM already fills the FP64 pipe.  Against every
+// candidate on 28 boxes: the sweeps within 3.5% of the fastest, 6% at two float64
+// ones (64^3, 200 x 131 x 67), k_div1 within 3%.  k_pred takes k_div1's constants,
+// though it does four times the work a cell, and is up to 17% (48^3) off its own
+// best; the float64 relativistic k_div1 up to 26% (32^3).  us per step at the fixed
+// 16 and at the model's choice: 2-D 128^2 float64 1326 and 369, 48^3 mixed 167 and
+// 112, 64^3 mixed 208 and 180, 512^2 mixed 124 and 109, 256^3 mixed 5144 and 5026.
 // Relativistic sweeps, fitted to 10 lengths of 16 boxes of the beam: a = 0.5
 // in float32 and 2 in float64, and c L more (c = 0.5, 0.75), since pencils
-// differ in their iterations and a long one finishes late; within 3% of the
-// fastest in float64, within 13% in float32 (6% on average).  us of the sweep along
+// differ in their iterations and a long one finishes late; within 6% of the
+// fastest in float64, within 11% in float32 (3% on average).  us of the sweep along
 // z at 8 cells, at 16 and at the choice: 64^3 mixed 376, 580, 285; 128^3 mixed
 // 1103, 1036, 1036; 64^3 float64 1068, 1280, 1068.
 // The Taub-Mathews gas in float32 (float64 iterations, whose number differs most
