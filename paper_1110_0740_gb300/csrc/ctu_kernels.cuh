@@ -244,7 +244,7 @@ __device__ __forceinline__ Where locate(const GroupTable &gt)
 }
 // The marching sweeps are latency bound: they are compiled for at least
 // CTU_MARCH_MINB resident blocks per SM (register cap 65536 / (BLOCK * MINB)),
-// the float relativistic ones for CTU_MARCH_MINB_SR (256^3 beam, z and y: 7.16
+// the float ones of the relativistic ideal gas for CTU_MARCH_MINB_SR (256^3 beam, z and y: 7.16
 // and 7.09 ms with three, 6.93 and 6.91 with four, 7.24 and 7.40 with five),
 // the float x sweep for CTU_SWEEPX_MINB (CTU_SWEEPX_MINB_PAR with the
 // parabolic terms, whose staging needs the registers of one block fewer).

@@ -73,7 +73,8 @@ inline void choose_segments(Group *g, int ng, int ndim, bool f64, bool rel, bool
     if (ndim < 2) return;
     for (int ring = 0; ring < 2; ++ring) {
         // the kernels' registers: 168 (three blocks), the float relativistic
-        // ones 128 (four), the float first-order ones about 95 (five)
+        // ones 128 (four; the Taub-Mathews ones three, fitted at four), the float
+        // first-order ones about 95 (five)
         const double fit = f64 ? 3.0 : ring ? 5.0 : rel ? 4.0 : 3.0;
         const double a = rel && !ring ? (f64 ? 2.0 : 0.5) : f64 && !rel ? 0.15 : 1.5;
         const double late = rel && !ring ? (f64 ? 0.75 : tm ? 2.0 : 0.5) : 0.0;

@@ -45,7 +45,10 @@ __device__ __forceinline__ bool d_pos(double x)
 {
     return (unsigned long long)(d_bits(x) - 1) < 0x7FF0000000000000ull;
 }
-__device__ __forceinline__ bool d_nonneg(double x) { return (unsigned long long)d_bits(x) <= (unsigned long long)D_INF || d_bits(x) == D_SIGN; }
+__device__ __forceinline__ bool d_nonneg(double x)
+{
+    return (unsigned long long)d_bits(x) <= (unsigned long long)D_INF || d_bits(x) == D_SIGN;
+}
 // |x| as an ordered integer, twice a magnitude, half of it
 __device__ __forceinline__ long long d_mag(double x) { return d_bits(x) & ~D_SIGN; }
 __device__ __forceinline__ long long d_twice(long long m) { return m >= D_ONE_EXP ? m + D_ONE_EXP : m << 1; }
