@@ -784,11 +784,11 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         return CTU_ECUDA;
     }
     ctx->tuning = true;
-    auto timed = [&](float &ms) -> ctu_status {
+    auto timed = [&](float &ms, int reps = 2) -> ctu_status {
         ctu_status r = step_common(ctx, U_in, U_out, stride, patches, npatch, d_dt_ch, nullptr, stream);
         if (r != CTU_OK) return r;
         float best = 1e30f;
-        for (int rep = 0; rep < 2; ++rep) {
+        for (int rep = 0; rep < reps; ++rep) {
             if (cudaEventRecord(e0, s) != cudaSuccess) return CTU_ECUDA;
             r = step_common(ctx, U_in, U_out, stride, patches, npatch, d_dt_ch, nullptr, stream);
             if (r != CTU_OK) return r;
@@ -801,11 +801,12 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         return CTU_OK;
     };
     // What an untuned step takes comes first (choose_segments; shapes tuned before
-    // start afresh): a shape is pinned only by a pair that beats it by 2%, more than
-    // two timings differ by, and the pins together only if their step is no slower.
-    // The candidates alone made small batches slower, since the rule takes segments
-    // down to one cell: 2-D 128^2 float64 177 us untuned and 264 tuned, 32^3 567 and
-    // 721.
+    // start afresh): a shape is pinned by a pair that beats it, and the pins are kept
+    // if the step with all of them beats the untuned one, each the best of six.  The
+    // candidates alone made small batches slower, since the rule takes segments down
+    // to one cell: 2-D 128^2 float64 177 us untuned and 264 tuned, 32^3 567 and 721.
+    // (A margin of 2% a shape lost the gains of a level's many shapes, each below it:
+    // a coarse step 11.20 ms against 11.02.)
     auto afresh = [&]() -> ctu_status {
         ctx->hpatch.clear();
         return bind_patches(ctx, patches, npatch, s);
@@ -815,7 +816,7 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
     for (const Group &G : ctx->groups) ctx->tune.erase(shape_key(G.n));
     st = afresh();
     float rule = 0.0f;
-    if (st == CTU_OK) st = timed(rule);
+    if (st == CTU_OK) st = timed(rule, 6);
     // coordinate descent over the shapes, largest first: for each, every
     // (tile width, segment) candidate with the other shapes fixed
     static const int kXw[] = {8, 16, 32};
@@ -826,7 +827,6 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         float bt = 0.0f;
         bool beaten = false;
         st = timed(bt);
-        bt *= 0.98f;
         const int nmax = std::max(G.n[0], std::max(G.n[1], G.n[2]));
         for (int xw : kXw) {
             if (xw > 8 && xw / 2 >= G.n[0] + 2) continue;  // wider than the patch
@@ -864,8 +864,8 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
     if (st == CTU_OK && other) {
         float t = 0.0f;
         st = afresh();
-        if (st == CTU_OK) st = timed(t);
-        if (st == CTU_OK && t > rule) {
+        if (st == CTU_OK) st = timed(t, 6);
+        if (st == CTU_OK && t >= rule) {
             for (const auto &k : pinned) ctx->tune.erase(k);
             st = afresh();
         }

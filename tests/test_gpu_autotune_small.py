@@ -23,8 +23,8 @@ def _time(ctx, U, Uo, P, d):
     return min(best)
 
 
-# A pair is kept only where it beats the default by 2%; two timings of one
-# configuration differ by less than 5%.
+# Pairs are kept only where their step beats the default's, each the best of six;
+# two such timings of one configuration differ by less than 5%.
 @pytest.mark.parametrize("n,ndim", [((128, 128, 1), 2), ((32, 32, 32), 3)], ids=["2d", "3d"])
 def test_tuned_is_no_slower(n, ndim):
     import torch
