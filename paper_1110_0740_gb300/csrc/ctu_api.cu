@@ -784,7 +784,7 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         return CTU_ECUDA;
     }
     ctx->tuning = true;
-    auto timed = [&](float &ms, int reps = 2) -> ctu_status {
+    auto timed = [&](float &ms, int reps = 4) -> ctu_status {
         ctu_status r = step_common(ctx, U_in, U_out, stride, patches, npatch, d_dt_ch, nullptr, stream);
         if (r != CTU_OK) return r;
         float best = 1e30f;
@@ -800,6 +800,8 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         ms = best;
         return CTU_OK;
     };
+    static const int kXw[] = {8, 16, 32};
+    static const int kSeg[] = {4, 8, 16, 32, 64};
     // What an untuned step takes comes first (choose_segments; shapes tuned before
     // start afresh): a shape is pinned by a pair that beats it, and the pins are kept
     // if the step with all of them beats the untuned one, each the best of six.  The
@@ -811,16 +813,19 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         ctx->hpatch.clear();
         return bind_patches(ctx, patches, npatch, s);
     };
-    std::vector<std::array<int, 3>> pinned;
+    // Where the default's own pair is one of the candidates it is pinned as such: what
+    // ctu_tile_params reports of a tuned shape then is what runs.
+    auto pin = [&](const int *n, int xw, int seg) {
+        if (std::find(std::begin(kSeg), std::end(kSeg), seg) != std::end(kSeg)) ctx->tune[shape_key(n)] = {xw, seg};
+    };
     bool other = false;  // a pin that is not the default's own pair
     for (const Group &G : ctx->groups) ctx->tune.erase(shape_key(G.n));
     st = afresh();
     float rule = 0.0f;
     if (st == CTU_OK) st = timed(rule, 6);
+    const std::vector<Group> plain(ctx->groups);
     // coordinate descent over the shapes, largest first: for each, every
     // (tile width, segment) candidate with the other shapes fixed
-    static const int kXw[] = {8, 16, 32};
-    static const int kSeg[] = {4, 8, 16, 32, 64};
     for (size_t g = 0; g < ctx->groups.size() && st == CTU_OK; ++g) {
         Group &G = ctx->groups[g];
         int bx = G.xw, bs = G.seg;
@@ -853,20 +858,16 @@ ctu_status ctu_autotune(ctu_ctx *ctx, const double *U_in, double *U_out, int64_t
         }
         G.xw = bx;
         G.seg = bs;
-        // the default's own pair, if it is one of the candidates, is kept as such: what
-        // ctu_tile_params reports of a tuned shape then is what runs
-        if (beaten || std::find(std::begin(kSeg), std::end(kSeg), bs) != std::end(kSeg)) {
-            ctx->tune[shape_key(G.n)] = {bx, bs};
-            pinned.push_back(shape_key(G.n));
-            other |= beaten;
-        }
+        pin(G.n, bx, bs);
+        other |= beaten;
     }
     if (st == CTU_OK && other) {
         float t = 0.0f;
         st = afresh();
         if (st == CTU_OK) st = timed(t, 6);
         if (st == CTU_OK && t >= rule) {
-            for (const auto &k : pinned) ctx->tune.erase(k);
+            for (const Group &G : plain) ctx->tune.erase(shape_key(G.n));
+            for (const Group &G : plain) pin(G.n, G.xw, G.seg);
             st = afresh();
         }
     }
